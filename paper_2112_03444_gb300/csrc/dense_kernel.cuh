@@ -48,10 +48,10 @@ __global__ void __launch_bounds__(kBlock, PREC == HC_PREC_DF ? 1 : kTrackMinBloc
   constexpr bool XDF = PREC == HC_PREC_DF;
   using RE = typename std::conditional<XDF, df, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L>();
+  const Group g = make_group<L, groups_meet(L, RING)>();
   const GroupMem sm = make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, 0,
                                         endgame_smem_bytes(L, MIXED), XDF ? 1 : 0);
-  DenseProblem<N, DEG, L> prob{&a, sm, g.mask};
+  DenseProblem<N, DEG, L> prob{&a, sm, g.meet};
   run_tracker<N, L, MIXED, DenseProblem<N, DEG, L>, RE, RING>(prob, a.c, g, sm);
 }
 

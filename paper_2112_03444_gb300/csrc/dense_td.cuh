@@ -75,7 +75,7 @@ struct DenseTD {
   cx<float>* Vf;   // the group's shared copies of the evaluation point (+ monomials)
   cx<double>* Vd;
   cx<df>* Vx;      // double-float kernels: the point as double-floats (+ monomials)
-  unsigned gmask;  // lanes of the group
+  unsigned gmask;  // lanes that evaluate together (Group meet)
 
   template <class R>
   __device__ __forceinline__ const cx<R>* dptr() const;

@@ -1298,6 +1298,7 @@ struct Bufs {
   int32_t* d_steps = nullptr;
   double* d_be = nullptr;
   unsigned long long* d_ctl = nullptr;  // kCtlWords control words (see kCtlBytes)
+  unsigned long long* hand = nullptr;   // mixed: hand-over links (LaunchCommon hand_list)
   unsigned long long* h_ctl = nullptr;  // pinned copy of d_ctl
   int64_t* esc_list = nullptr;
   int64_t* dup_list = nullptr;
@@ -1364,6 +1365,10 @@ hc_status alloc_scratch(hc_problem* p, int64_t n_inst, Bufs& B, A&& alloc) {
   }
   if ((rc = alloc(kCtlBytes, &q)) != HC_OK) return rc;
   B.d_ctl = (unsigned long long*)q;
+  if (mixed) {
+    if ((rc = alloc(sizeof(unsigned long long) * items, &q)) != HC_OK) return rc;
+    B.hand = (unsigned long long*)q;
+  }
   if (escalate) {
     if ((rc = alloc(sizeof(int64_t) * items, &q)) != HC_OK) return rc;
     B.esc_list = (int64_t*)q;
@@ -1457,6 +1462,7 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   cm.x32_out = B.x32;
   cm.dup_list = B.dup_list;
   cm.dup_count = B.d_ctl + 7;
+  cm.hand_list = B.hand;
   // Re-tracking tiers.  Colliding endpoints (path jumps, found by the
   // duplicate check) and FP32-tier failures other than step-size ones
   // (divergence, non-finite state, failed refinement: dup_list, ctl[7]) run

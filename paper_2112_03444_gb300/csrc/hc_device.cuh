@@ -98,14 +98,22 @@ struct Group {
   int gl;          // lane index inside the group (row index)
   int wl;          // lane index inside the warp
   unsigned mask;   // lanes of this group
+  unsigned meet;   // lanes that run the evaluation and the solve together
 };
 
-template <int L>
+// MEET: the warp's groups run the evaluation and the solve in step (all lanes
+// of the warp pass there equally often), so that the code there can use
+// warp-wide masks.  A warp instruction with a mask that differs between the
+// groups runs once per group and leaves the groups apart: with group masks in
+// the solve, a third to a half of the lanes were idle (cubic n = 5: 15 to 24
+// of 32 active per instruction).
+template <int L, bool MEET = false>
 __device__ __forceinline__ Group make_group() {
   Group g;
   g.wl = threadIdx.x & 31;
   g.gl = g.wl & (L - 1);
   g.mask = (L == 32) ? 0xffffffffu : (((1u << L) - 1u) << (g.wl & ~(L - 1)));
+  g.meet = MEET ? 0xffffffffu : g.mask;
   return g;
 }
 
@@ -114,10 +122,24 @@ __device__ __forceinline__ cx<R> shfl(unsigned mask, cx<R> v, int src) {
   return {__shfl_sync(mask, v.re, src), __shfl_sync(mask, v.im, src)};
 }
 
+// max over the group of an unsigned integer.  MEET: by all lanes of the warp
+// together.
+template <int L, bool MEET>
+__device__ __forceinline__ unsigned gmaxu(const Group& g, unsigned v) {
+  if constexpr (L == 32 || !MEET) {
+    return __reduce_max_sync(L == 32 ? 0xffffffffu : g.mask, v);
+  } else {
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+  }
+}
 // max over the group of a non-negative float (NaN compares above everything)
+__device__ __forceinline__ unsigned max_key(float v) {
+  return __float_as_uint(fmaxf(v, 0.0f)) | (isnan(v) ? 0x7fc00000u : 0u);
+}
 __device__ __forceinline__ float gmaxf(const Group& g, float v) {
-  unsigned b = __reduce_max_sync(g.mask, __float_as_uint(fmaxf(v, 0.0f)) | (isnan(v) ? 0x7fc00000u : 0u));
-  return __uint_as_float(b);
+  return __uint_as_float(__reduce_max_sync(g.mask, max_key(v)));
 }
 __device__ __forceinline__ bool gany(const Group& g, bool v) {
   return __reduce_or_sync(g.mask, v ? 1u : 0u) != 0u;
@@ -156,7 +178,7 @@ __device__ __forceinline__ R gsum(const Group& g, R v) {
 // On return lane i with i < N holds in col the column it pivoted on and in
 // sol[r] the solution component x[col] of right-hand side r.  Returns false
 // if a pivot was zero or non-finite (the caller rejects the step).
-template <int N, int NR, class R>
+template <int N, int NR, class R, int L = 32, bool MEET = false>
 __device__ __forceinline__ bool gj_solve(const Group& g, cx<R> (&a)[N + NR], cx<R> (&sol)[NR],
                                          int& col, cx<R>* pv) {
   constexpr int W = N + NR;
@@ -175,7 +197,7 @@ __device__ __forceinline__ bool gj_solve(const Group& g, cx<R> (&a)[N + NR], cx<
     inv = crecip(a[k]);
     const float m = (float)cabs1(a[k]);
     const unsigned key = used ? 0u : ((__float_as_uint(m) & ~31u) | (unsigned)(31 - g.wl));
-    kmax = __reduce_max_sync(g.mask, key);
+    kmax = MEET ? gmaxu<L, MEET>(g, key) : __reduce_max_sync(g.mask, key);
   };
   cx<R> inv;
   unsigned kmax;
@@ -204,7 +226,7 @@ __device__ __forceinline__ bool gj_solve(const Group& g, cx<R> (&a)[N + NR], cx<
       dinv = inv;
       col = k;
     }
-    __syncwarp(g.mask);
+    __syncwarp(g.meet);
     cx<R> row_p[W];  // the pivot row, columns k .. W-1 (slot k: 1/pivot)
     if constexpr (sizeof(R) == 4) {
 #pragma unroll

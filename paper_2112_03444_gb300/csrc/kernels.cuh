@@ -96,6 +96,9 @@ struct LaunchCommon {
   int spread;                   // first round of items round-robin over the blocks (one
                                 // per block before any second), then the queue: a short
                                 // list of FP64-heavy paths lands on as many SMs as it can
+  // Links of the mixed batch kernels' hand-over lists (tracker.cuh), one word
+  // per item, written before it is read.
+  unsigned long long* hand_list;
   // Resident launches (hc_stream): items come from a ring of instance slots
   // that the host fills while the launch runs.  Ticket q (claimed from
   // *queue only while q < *ring_tail, which the host's staging stream writes

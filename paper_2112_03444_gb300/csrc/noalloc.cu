@@ -32,9 +32,14 @@
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = size_t(16) << 20;  // 16 MiB per device
+// behind it the mixed kernels' hand-over links, 8 bytes per path: the encoded
+// coefficients of a batch that fits the scratch take at least 2.3 times that
+// (cubic n = 8: 6561 paths against 121,728 bytes per system, rounded up here)
+constexpr size_t kNoAllocHandBytes = size_t(8) << 20;
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes +
+                                                                kNoAllocHandBytes];
 
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
@@ -235,6 +240,11 @@ extern "C" hc_status hc_track_dense_noalloc(int32_t n, int32_t degree, const dou
     hc::set_last_error(msg);
     return HC_ERR_INVALID;
   }
+  const size_t hand_b = mixed ? sizeof(unsigned long long) * (size_t)items : 0;
+  if (hand_b > kNoAllocHandBytes) {  // cannot be for a batch that fits above
+    hc::set_last_error("hc_track_dense_noalloc: batch has too many paths");
+    return HC_ERR_INVALID;
+  }
   void* base = nullptr;
   hc_status rc = scratch_address(&base);
   if (rc != HC_OK) return rc;
@@ -258,6 +268,8 @@ extern "C" hc_status hc_track_dense_noalloc(int32_t n, int32_t degree, const dou
   double* t_io = escalate ? reinterpret_cast<double*>(p) : nullptr;
   p += tio_b;
   float2* x32 = escalate ? reinterpret_cast<float2*>(p) : nullptr;
+  unsigned long long* hand = reinterpret_cast<unsigned long long*>(
+      static_cast<unsigned char*>(base) + kNoAllocScratchBytes);
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 #define NA_CUDA(call)                                                                   \
@@ -295,6 +307,7 @@ extern "C" hc_status hc_track_dense_noalloc(int32_t n, int32_t degree, const dou
   a.c.x32_out = x32;
   a.c.dup_list = escalate ? dup : nullptr;
   a.c.dup_count = ctl + 7;
+  a.c.hand_list = hand;
   a.D32 = reinterpret_cast<const hc::cx<float>*>(D32);
   a.D64 = reinterpret_cast<const hc::cx<double>*>(D64);
   a.Ddf = reinterpret_cast<const hc::cx<hc::df>*>(Ddf);

@@ -120,12 +120,12 @@ struct TermEval {
       return Vd;
   }
 
-  // p(t) into V (each lane a share), then wait for the group.  FP64:
+  // p(t) into V (each lane a share), then wait for `lanes`.  FP64:
   // (1-t) p0 + t p1 from the inputs; FP32: p0 + t dp from the FP32 copies;
   // double-float: p0 + t dp from the double-float copies, and the point
   // (which the tracker keeps in FP64 in Vd) split into double-floats.
   template <class R>
-  __device__ __forceinline__ void put_params(R t) const {
+  __device__ __forceinline__ void put_params(R t, unsigned lanes) const {
     const int P = a->P, LS = a->ls;
     if constexpr (std::is_same<R, float>::value) {
       for (int l = g.gl; l < P; l += L)
@@ -142,7 +142,7 @@ struct TermEval {
         Vd[LS + 1 + l] = mk<double>((1.0 - t) * q0.x + t * q1.x, (1.0 - t) * q0.y + t * q1.y);
       }
     }
-    __syncwarp(g.mask);
+    __syncwarp(lanes);
   }
 
   // One term of D factors: add its value to h and its derivatives to the
@@ -197,7 +197,7 @@ struct TermEval {
   template <class R>
   __device__ __forceinline__ void eval(const cx<R> (&)[N], int i, R t, R, cx<R> (&row)[N + 1],
                                        cx<R>& H, cx<R>& Ht) const {
-    put_params<R>(t);
+    put_params<R>(t, g.meet);
     const cx<R>* V = vptr<R>();
     const int rr = i & (ROWL - 1), part = i / ROWL;  // row, and share of the term slots
     const int ii = rr < N ? rr : 0;
@@ -251,7 +251,7 @@ struct TermEval {
   template <bool SCALE, int EP = 1>
   __device__ __forceinline__ void residual64(const cx<double>*, int i, double t, double,
                                              cx<double>& H, double& sc) const {
-    put_params<double>(t);
+    put_params<double>(t, g.mask);
     const int rr = i & (ROWL - 1), part = i / ROWL;
     const int ii = rr < N ? rr : 0;
     cx<double> h = czero<double>();
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kBlock) term_param_kernel(const __grid_constan
   constexpr bool XDF = PREC == HC_PREC_DF;
   using RE = typename std::conditional<XDF, df, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L>();
+  const Group g = make_group<L, groups_meet(L, RING)>();
   const GroupMem sm = make_group_mem<L>(smem, a.extra, term_acc_bytes<N, MIXED, L>(),
                                         endgame_smem_bytes(L, MIXED), XDF ? 1 : 0);
   TermProblem<N, L, MIXED> prob{&a, g, sm};

@@ -9,7 +9,7 @@
 // accept iff Newton converges within max_newton iterations and its first
 // correction is small; double dt after grow_after accepts; halve on reject.
 //
-// Code shape.  Every phase of the method needs the same work item: evaluate
+// Code shape (of each loop, see run_tracker).  Every phase of the method needs the same work item: evaluate
 // row i of [dH/dx | rhs] at some point and time, solve, and scatter the
 // solution.  A lane group therefore runs ONE loop around ONE copy of the
 // (fully unrolled) evaluation and solve, driven by a small state machine:
@@ -85,6 +85,61 @@ __device__ __forceinline__ void load_vec(const cx<S>* buf, cx<R> (&x)[N]) {
 // (kernels with cooperative residuals, which keep the warp together)
 enum : int { M_RK = 0, M_NEWTON = 1, M_REFINE = 2, M_COND = 3, M_DONE = 4, M_FETCH = 5, M_IDLE = 6 };
 
+// Kernels whose warps hold several groups and keep them in step (see
+// make_group); the groups of a resident launch wait for work on their own.
+__host__ __device__ constexpr bool groups_meet(int L, bool ring) { return !ring && L < 32; }
+
+// Phases of the mixed kernels: the whole path in one loop (resident launches),
+// its FP32 phase only, or everything after it.
+enum : int { P_WHOLE = 0, P_LOW = 1, P_HIGH = 2 };
+
+// Hand-over from the low to the high phase: a list per block, its head in
+// shared memory, the links in hand_list (one word per item).  Entry: item + 1
+// in 40 bits (0: end of the list), the reason in 2 and the accepted steps in a
+// row in 22 (saturated: a path takes at most about 1e5 steps, and the count
+// starts again every grow_after of them).
+enum : int {
+  H_GOES_ON = 0,  // end of the FP32 phase, or its step budget: dt stays
+  H_REFINE = 1,   // t = 1 reached
+  H_DONE = 2,     // failed or diverged: status in status_out
+  H_STALLED = 3   // steps below dt_min_fp32: goes on with that dt
+};
+__device__ __forceinline__ unsigned long long hand_entry(int64_t item, int code, int consec) {
+  return (unsigned long long)(item + 1) | (unsigned long long)code << 40 |
+         (unsigned long long)min(consec, (1 << 22) - 1) << 42;
+}
+__device__ __forceinline__ int64_t hand_item(unsigned long long e) {
+  return (int64_t)(e & ((1ull << 40) - 1)) - 1;
+}
+__device__ __forceinline__ int hand_code(unsigned long long e) { return (int)(e >> 40) & 3; }
+__device__ __forceinline__ int hand_consec(unsigned long long e) { return (int)(e >> 42); }
+// Both retry only when another group of the block changed the head between
+// the read and the exchange.  An item is on the list at most once in a launch,
+// so a head that compares equal still has the same link.
+__device__ __forceinline__ void hand_push(const LaunchCommon& c, unsigned long long* head,
+                                          unsigned long long e) {
+  unsigned long long h = *reinterpret_cast<volatile unsigned long long*>(head);
+  for (;;) {
+    __stcg(c.hand_list + hand_item(e), h);
+    __threadfence_block();
+    const unsigned long long was = atomicCAS(head, h, e);
+    if (was == h) break;
+    h = was;
+  }
+}
+__device__ __forceinline__ unsigned long long hand_pop(const LaunchCommon& c,
+                                                       unsigned long long* head) {
+  unsigned long long h = *reinterpret_cast<volatile unsigned long long*>(head);
+  while (h != 0) {
+    const unsigned long long next = __ldcg(c.hand_list + hand_item(h));
+    const unsigned long long was = atomicCAS(head, h, next);
+    if (was == h) break;
+    h = was;
+  }
+  __threadfence_block();
+  return h;
+}
+
 // Shared memory of one lane group: pv = two pivot-row buffers of the solve,
 // acc = evaluator accumulators (term evaluator only), vd = high-precision
 // copy of the evaluation point (complex FP64 in the all-FP64 kernels,
@@ -104,6 +159,7 @@ struct GroupMem {
   cx<df>* vx;      // double-float kernels: the evaluator's double-float copy of
                    // vd (L + extra entries), 16-byte aligned; nullptr otherwise
   int stride;      // bytes from one group's memory to the next group's
+  unsigned long long* hand;  // the block's hand-over head (mixed batch kernels)
 };
 
 template <int L>
@@ -114,6 +170,9 @@ __device__ __forceinline__ GroupMem make_group_mem(unsigned char* smem, int extr
   unsigned char* b = smem + (threadIdx.x / L) * stride;
   GroupMem m;
   m.stride = stride;
+  // the 16 bytes by which the stride passes a multiple of 128 are not used
+  // otherwise: those of the block's first group
+  m.hand = reinterpret_cast<unsigned long long*>(smem + stride - 16);
   m.pv = b;
   b += 32 * (L + 2);
   m.acc = b;
@@ -177,9 +236,12 @@ __device__ __forceinline__ cx<double> hermite_at_zero(double wb, cx<double> xb, 
 // FP64 kernels.  RING: the resident launch of a stream (hc_stream), whose
 // items come from the host-filled ring (LaunchCommon ring_*); compiled only
 // into the kernels the streams use.
-template <int N, int L, bool MIXED, class PROB, class RE = double, bool RING = false>
-__device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon& c,
-                                            const Group& g, const GroupMem& sm) {
+template <int N, int L, bool MIXED, class PROB, class RE = double, bool RING = false,
+          int PHASE = P_WHOLE>
+__device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& c, const Group& g,
+                                          const GroupMem& sm) {
+  static_assert(PHASE == P_WHOLE || (MIXED && !RING), "phases: mixed kernels of a batch");
+  constexpr bool LOW = PHASE == P_LOW;
   using R = typename std::conditional<MIXED, float, RE>::type;
   using HOM = decltype(prob.hom(0));
   // double-float kernels: their Newton corrector takes its residual in FP64
@@ -196,7 +258,11 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
   // The resident-launch kernels (whose groups wait for tickets on their own)
   // compute the same partial sums in the same order group by group (EP).
   constexpr bool COOP_EVAL = MIXED && HOM::kCoop;
-  constexpr bool COOP = COOP_EVAL && !RING;
+  constexpr bool COOP = COOP_EVAL && !RING && !LOW;
+  // Warps with several groups meet once per iteration and leave together (a
+  // group out of work is M_IDLE until then): without that point the groups
+  // drift apart and each runs the evaluation and the solve on its own.
+  constexpr bool MEET = groups_meet(L, RING);
   constexpr int EP = COOP_EVAL ? 32 / L : 1;
   const DevSettings& s = c.s;
   cx<R>* sb = reinterpret_cast<cx<R>*>(sm.sb);
@@ -226,11 +292,12 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
   (void)ticket;
   cx<double> xd = czero<double>();  // FP64 state
   cx<float> xf = czero<float>();    // FP32 state
-  bool hi = !MIXED;                 // the state lives in xd rather than xf
+  bool hi = !MIXED || PHASE == P_HIGH;  // the state lives in xd rather than xf
   // t, dt, h, t1: FP64-state phase; tf, dtf, hf, t1f: FP32 phase
   double t = 0.0, dt = 0.0, h = 0.0, t1 = 0.0;
   float tf = 0.f, dtf = 0.f, hf = 0.f, t1f = 0.f;
   int consec = 0, nacc = 0, nrej = 0, nnewt = 0, status = 0;
+  int counted = 0;  // steps of the path already added to *step_total (P_HIGH)
   int mode = M_FETCH, stage = 0, it = 0;
   cx<R> kprev = czero<R>(), ksum = czero<R>();
   cx<float> xpf = czero<float>();   // corrector iterate (FP32 state)
@@ -258,8 +325,29 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
   cx<R> sol[1];
   int col;
 
-  // hi is constant true in the plain FP64 kernel; say so to the compiler
-  auto HI = [&]() { return !MIXED || hi; };
+  // hi is constant in the plain FP64 kernel and in a single phase; say so to
+  // the compiler
+  auto HI = [&]() { return !MIXED || PHASE == P_HIGH || (!LOW && hi); };
+  // P_LOW: the path leaves the FP32 phase.  Its state goes into the item's own
+  // output slots, which the high phase overwrites with the results: FP32 point
+  // and (tf, dtf) in x_out (16 N bytes hold 8 N + 8), counters in steps_out;
+  // then the item is published on the hand-over list.
+  auto hand_over = [&](int code) {
+    float2* slot = reinterpret_cast<float2*>(c.x_out + item * (2 * N));
+    if (act) slot[g.gl] = make_float2(xf.re, xf.im);
+    if (g.gl == 0) {
+      slot[N] = make_float2(tf, dtf);
+      c.steps_out[item * 3 + 0] = nacc;
+      c.steps_out[item * 3 + 1] = nrej;
+      c.steps_out[item * 3 + 2] = nnewt;
+      if (code == H_DONE) c.status_out[item] = (uint8_t)status;
+      if (c.step_budget) atomicAdd(c.step_total, (unsigned long long)(nacc + nrej));
+    }
+    __threadfence_block();
+    __syncwarp(g.mask);
+    if (g.gl == 0) hand_push(c, sm.hand, hand_entry(item, code, consec));
+    mode = M_FETCH;
+  };
   // this lane's entry of the high-precision point copy, as double-floats
   // (as_df) or complex FP64
   auto put_hi = [&](const cx<double>& v, bool as_df) {
@@ -297,6 +385,10 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
     hi = true;
   };
   auto enter_refine = [&]() {
+    if constexpr (LOW) {
+      hand_over(H_REFINE);
+      return;
+    }
     if (!HI()) xd = cvt<double>(xf);
     hi = true;
     mode = M_REFINE;
@@ -377,20 +469,28 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       }
     } else {
       dtf *= 0.5f;
-      if (dtf < dt_min32f) {
-        // FP32 cannot resolve this stretch of the path (its corrector stalls
-        // at the FP32 noise floor): continue from the last accepted point
-        // with the FP64 state and FP64 residuals instead of failing the path.
-        promote(s.dt_min_fp32);
+      // below dt_min_fp32, FP32 cannot resolve this stretch of the path (its
+      // corrector stalls at the FP32 noise floor): continue from the last
+      // accepted point with the FP64 state and FP64 residuals instead of
+      // failing the path
+      if (LOW && dtf < dt_min32f) {
+        hand_over(H_STALLED);
+      } else {
+        if (dtf < dt_min32f) promote(s.dt_min_fp32);
+        begin_step();
       }
-      begin_step();
     }
   };
 
 #pragma unroll 1
   for (;;) {
     // ---- 0. retire the finished path and refill the group with the next one
-    if (mode == M_DONE) {
+    // (no `continue` and no `break` inside a mode's branch: a warp whose groups
+    // part there is put together again only behind both, that is, behind the
+    // evaluation and the solve)
+    if constexpr (LOW)
+      if (mode == M_DONE) hand_over(H_DONE);
+    if (!LOW && mode == M_DONE) {
       if (!hi) xd = cvt<double>(xf);
       if ((status & 0x7f) != ST_FINITE && status != ST_FAIL_NAN && gany(g, act && !cfinite(xd)))
         status = ST_FAIL_NAN;
@@ -408,7 +508,8 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       if (g.gl == 0) {
         c.status_out[item] = (uint8_t)status;
         if (c.be_out) c.be_out[item] = (double)be;
-        if (c.step_budget) atomicAdd(c.step_total, (unsigned long long)(nacc + nrej));
+        if (c.step_budget)
+          atomicAdd(c.step_total, (unsigned long long)(nacc + nrej - counted));
         if (MIXED) {
           c.steps_out[item * 3 + 0] = nacc;
           c.steps_out[item * 3 + 1] = nrej;
@@ -497,6 +598,50 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       (void)ld_acquire_gpu(c.ring_tail);  // every lane: the slot's inputs are visible
       item = (int64_t)(ticket % c.ring_items);
     }
+    if constexpr (PHASE == P_HIGH) {
+      if (mode == M_FETCH && c.hand_list && !c.start_hi) {
+        // the next path the low phase has handed over; with none on the list
+        // the group is done, since whoever hands one over later comes here
+        // after it (see run_tracker)
+        unsigned long long e = 0;
+        if (g.gl == 0) e = hand_pop(c, sm.hand);
+        e = __shfl_sync(g.mask, e, leader);
+        if (e == 0) {
+          if constexpr (MEET)
+            mode = M_IDLE;
+          else
+            break;
+        } else {
+          item = hand_item(e);
+          const int code = hand_code(e);
+          inst_cur = item / c.paths;
+          hom = prob.hom(inst_cur);
+          hom.init(g);
+          const float2* slot = reinterpret_cast<const float2*>(c.x_out + item * (2 * N));
+          const float2 v = act ? __ldcg(slot + g.gl) : make_float2(0.f, 0.f);
+          const float2 tt = __ldcg(slot + N);
+          xd = mk<double>((double)v.x, (double)v.y);
+          t = (double)tt.x;
+          dt = code == H_STALLED ? s.dt_min_fp32 : (double)tt.y;
+          consec = hand_consec(e);
+          nacc = __ldcg(c.steps_out + item * 3 + 0);
+          nrej = __ldcg(c.steps_out + item * 3 + 1);
+          nnewt = __ldcg(c.steps_out + item * 3 + 2);
+          counted = nacc + nrej;
+          status = code == H_DONE ? (int)__ldcg(c.status_out + item) : 0;
+          res64 = false;
+          be = 0.f;
+          eg_landing = eg_pending = eg_have = eg_sing = false;
+          __syncwarp(g.mask);
+          if (code == H_DONE)
+            mode = M_DONE;
+          else if (code == H_REFINE)
+            enter_refine();
+          else
+            begin_step();
+        }
+      }
+    }
     if (mode == M_FETCH) {
       bool stop = false;  // no further path for this group
       if (c.step_budget && !c.items) {
@@ -520,7 +665,7 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       }
       if (!RING && !stop) stop = (int64_t)q >= total;
       if (stop) {
-        if constexpr (COOP)
+        if constexpr (MEET)
           mode = M_IDLE;
         else
           break;
@@ -545,12 +690,12 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
           }
         }
         xf = cvt<float>(xd);
-        hi = !MIXED || c.start_hi;
+        hi = !MIXED || PHASE == P_HIGH || c.start_hi;
         t = t0 > 0.0 ? t0 : 0.0;
         dt = s.dt_init;
         tf = (float)t;
         dtf = (float)s.dt_init;
-        consec = nacc = nrej = nnewt = status = 0;
+        consec = nacc = nrej = nnewt = status = counted = 0;
         res64 = false;
         be = 0.f;
         // endgame: the first sample time after the start point
@@ -575,11 +720,13 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       if (nacc + nrej >= s.max_steps) {
         status = ST_FAIL_MAXSTEPS;
         mode = M_DONE;
-        continue;
-      }
-      if (!HI() && nacc + nrej >= s.max_steps_fp32) {  // FP32 step budget spent
-        promote((double)dtf);
-        begin_step();
+      } else if (!HI() && nacc + nrej >= s.max_steps_fp32) {  // FP32 step budget spent
+        if constexpr (LOW) {
+          hand_over(H_GOES_ON);
+        } else {
+          promote((double)dtf);
+          begin_step();
+        }
       }
     }
 
@@ -621,7 +768,7 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
         omt = (R)(1.f - t1f);
         if (act) sm.vf[g.gl] = xpf;
       }
-    } else {  // M_REFINE, M_COND (M_IDLE: nothing to evaluate): at the endpoint, t = 1
+    } else if constexpr (!LOW) {  // M_REFINE, M_COND (M_IDLE: nothing to evaluate): at t = 1
       need64 = (mode == M_REFINE);
       // COOP: the backward error of a refined endpoint comes with the first
       // condition pass (the same point)
@@ -630,21 +777,22 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       if (MIXED) res_code = need64 ? 1 : be_now ? 3 : 0;
       if (act) sm.vf[g.gl] = cvt<float>(xd);
     }
-    __syncwarp(g.mask);
+    __syncwarp(g.meet);
     if constexpr (MIXED) {
       load_vec<N, float, float>(sm.vf, x);
     } else {
       load_vec<N, double, R>(sm.vd, x);
     }
 
-    if constexpr (COOP) {
-      // The loop's one warp-wide meeting point: leave together once every
-      // group is idle, else compute the groups' residuals one group at a
-      // time with all lanes of the warp.  A lane of the group served keeps
-      // its row's residual (FP32-rounded) and scale in its own entry of the
-      // group's scatter buffer, which is free until the solve.
+    if constexpr (MEET) {
       const unsigned live = __ballot_sync(0xffffffffu, g.gl == 0 && mode != M_IDLE);
       if (live == 0u) break;
+    }
+    if constexpr (COOP) {
+      // Here the warp computes the groups' residuals one group at a time with
+      // all its lanes.  A lane of the group served keeps its row's residual
+      // (FP32-rounded) and scale in its own entry of the group's scatter
+      // buffer, which is free until the solve.
       const unsigned want = __ballot_sync(0xffffffffu, g.gl == 0 && res_code != 0);
       if (want != 0u) {
         __syncwarp(0xffffffffu);  // the groups' point copies, before other groups read them
@@ -689,7 +837,7 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
       hom.template eval<R>(x, g.gl, ter, omt, row, H, Ht);
       if (mode == M_RK) {
         row[N] = -Ht;
-      } else if (mode == M_COND) {
+      } else if (!LOW && mode == M_COND) {
         if (stage == 0) {  // first column pass: 1-norm of the matrix
           float an = 0.f;
 #pragma unroll
@@ -700,7 +848,7 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
         // unit vector e_stage (on every replica of row stage)
         const int grow = g.gl & (HOM::ROWL - 1);
         row[N] = mk<R>((grow < N && grow == stage) ? R(1) : R(0), R(0));
-      } else if (need64) {
+      } else if (!LOW && need64) {
         if constexpr (COOP) {
           const float4 v = reinterpret_cast<const float4*>(sm.sb)[g.gl];
           row[N] = mk<R>(-v.x, -v.y);
@@ -726,27 +874,44 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
                                                        reinterpret_cast<cx<R>*>(sm.pv),
                                                        reinterpret_cast<cx<R>*>(sm.sb));
     else
-      sok = gj_solve<N, 1, R>(g, row, sol, col, reinterpret_cast<cx<R>*>(sm.pv));
+      sok = gj_solve<N, 1, R, L, MEET>(g, row, sol, col, reinterpret_cast<cx<R>*>(sm.pv));
     if (col >= 0) sb[col] = sol[0];
-    __syncwarp(g.mask);
+    __syncwarp(g.meet);
     const cx<R> d = act ? sb[g.gl] : czero<R>();
+    // the new iterate of a Newton step and the sizes (inf-norms) of it and of
+    // the step, reduced outside the mode branches, where all groups are
+    cx<double> xnd = czero<double>();
+    cx<float> xnf_ = czero<float>();
+    if (mode == M_NEWTON || (!LOW && mode == M_REFINE)) {
+      if (HI()) {
+        xnd = (!LOW && mode == M_REFINE ? xd : xpd) + cvt<double>(d);
+        xnf_ = cvt<float>(xnd);
+      } else {
+        xnf_ = xpf + cvt<float>(d);
+      }
+    }
+    const float xn_all = sqrt_approx(
+        __uint_as_float(gmaxu<L, MEET>(g, max_key(act ? cnorm2(xnf_) : 0.f))));
+    const float dn_all = sqrt_approx(
+        __uint_as_float(gmaxu<L, MEET>(g, max_key(act ? (float)cnorm2(d) : 0.f))));
 
     // ---- 3. state machine
     if (mode == M_RK) {
+      bool ended = false;
       if constexpr (!MIXED) {
         // stage 1 at a sample point gives its dx/dt
         if (stage == 0 && eg_pending) {
           eg_pending = false;
           if (sok && eg_sample(cvt<double>(d))) {
             eg_finish();
-            continue;
+            ended = true;
           }
         }
       }
       step_ok = step_ok && sok;
       kprev = d;
       ksum = ksum + ((stage == 0 || stage == 3) ? R(1) : R(2)) * d;
-      if (++stage == 4) {
+      if (!ended && ++stage == 4) {
         if (!step_ok) {
           reject();
         } else {
@@ -759,17 +924,12 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
         }
       }
     } else if (mode == M_NEWTON) {
-      float xn2;
-      if (HI()) {
-        xpd = xpd + cvt<double>(d);
-        xn2 = gmaxf(g, act ? cnorm2(cvt<float>(xpd)) : 0.f);
-      } else {
-        xpf = xpf + cvt<float>(d);
-        xn2 = gmaxf(g, act ? cnorm2(xpf) : 0.f);
-      }
+      if (HI())
+        xpd = xnd;
+      else
+        xpf = xnf_;
       ++nnewt;
-      const float xn = sqrt_approx(xn2);
-      const float dn = sqrt_approx(gmaxf(g, act ? (float)cnorm2(d) : 0.f));
+      const float xn = xn_all, dn = dn_all;
       const bool bad = !sok || !(dn <= 3.0e38f) || !(xn <= 3.0e38f) ||
                        (it == 0 && dn > (HI() ? corr64 : corr32) * (1.f + xn));
       if (!bad && dn <= (HI() ? tol64 : tol32) * (1.f + xn)) {
@@ -795,22 +955,25 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
         } else if (at_end) {
           enter_refine();
         } else {
-          if (!HI() && tf >= tAf) promote((double)dtf);  // enter the FP64-state phase
-          if (eg_on && eg_landing) {  // the step ended on a sample time
-            eg_pending = true;
-            eg_s_sample = eg_s;
-            eg_s *= s.eg_ratio;
-            ++eg_next;
+          if (LOW && tf >= tAf) {  // the FP64-state phase begins here
+            hand_over(H_GOES_ON);
+          } else {
+            if (!HI() && tf >= tAf) promote((double)dtf);  // enter the FP64-state phase
+            if (eg_on && eg_landing) {  // the step ended on a sample time
+              eg_pending = true;
+              eg_s_sample = eg_s;
+              eg_s *= s.eg_ratio;
+              ++eg_next;
+            }
+            begin_step();
           }
-          begin_step();
         }
       } else if (bad || ++it >= ((MIXED && HI()) ? s.max_newton_ir : s.max_newton)) {
         reject();
       }
-    } else if (mode == M_REFINE) {
-      const cx<double> xnew = xd + cvt<double>(d);
-      const float dn = sqrt_approx(gmaxf(g, act ? (float)cnorm2(d) : 0.f));
-      const float xnn = sqrt_approx(gmaxf(g, act ? cnorm2(cvt<float>(xnew)) : 0.f));
+    } else if (!LOW && mode == M_REFINE) {
+      const cx<double> xnew = xnd;
+      const float dn = dn_all, xnn = xn_all;
       const bool bad = !sok || !(dn <= 3.0e38f) || !(xnn <= 3.0e38f);
       if (!bad && !eg_sing) xd = xnew;
       if (bad || eg_sing || dn <= (float)s.refine_tol * (1.f + xnn) || ++it >= s.refine_iters) {
@@ -859,10 +1022,10 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
           }
         }
       }
-    } else if (mode == M_COND && COOP && stage == 0 && be_bad) {
+    } else if (!LOW && mode == M_COND && COOP && stage == 0 && be_bad) {
       status = ST_FAIL_REFINE;  // the refined endpoint failed the backward-error test
       mode = M_DONE;
-    } else if (mode == M_COND) {
+    } else if (!LOW && mode == M_COND) {
       if (!sok) cond_inorm = INFINITY;
       cond_inorm =
           fmaxf(cond_inorm, gsum<L, float>(g, (act && col >= 0) ? cabs2(cvt<float>(d)) : 0.f));
@@ -880,6 +1043,43 @@ __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon
         mode = M_DONE;
       }
     }
+  }
+}
+
+// The persistent loop of a tracking kernel.  The mixed kernels with several
+// paths per warp run it as two loops one after the other: the FP32 phases of
+// all paths, then what is left of each (FP64 state, refinement,
+// classification).  What bounds these kernels is instruction fetch: measured on
+// GB300, straight-line code issues at full rate while the code a warp cycles
+// through fits 32 KB, at a third of it (a half with four warps per scheduler)
+// up to 128 KB, and at a fifth beyond.  One loop over all phases cycles through
+// about 60 KB, since among the paths of a warp some is always near its end; the
+// FP32 loop alone about fits.  Together with the warp-wide masks (make_group)
+// and branches that end where they began, the tracking launches went, in ms,
+// cubic n = 8 (16 systems) 40.2 -> 34.5, quadratic n = 12 (16) 33.7 -> 31.6, one
+// quadratic n = 6 system 1.20 -> 0.65, 4-view triangulation (600 scenes)
+// 372 -> 331, P3P (3000) 18.4 -> 14.6.  One path per warp keeps the single loop:
+// its items are few and long, and the second loop would wait for the warp's own
+// paths (trifocal, 4 scenes: 184 -> 206 with two loops).
+//
+// The second loop waits for nothing: a path goes onto its block's hand-over
+// list from its warp's first loop, so the warp that handed over last still has
+// its second loop ahead, where it takes every path the others left.  (One list
+// for the whole grid loses more to the contention on its head than its balance
+// gives: cubic n = 8, 40 -> 190 ms with a compare-and-swap per path.)
+template <int N, int L, bool MIXED, class PROB, class RE = double, bool RING = false>
+__device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon& c,
+                                            const Group& g, const GroupMem& sm) {
+  if constexpr (MIXED && groups_meet(L, RING)) {
+    if (!c.start_hi) {
+      if (threadIdx.x == 0) *sm.hand = 0;
+      __syncthreads();
+      run_phase<N, L, MIXED, PROB, RE, RING, P_LOW>(prob, c, g, sm);
+      __syncwarp();
+    }
+    run_phase<N, L, MIXED, PROB, RE, RING, P_HIGH>(prob, c, g, sm);
+  } else {
+    run_phase<N, L, MIXED, PROB, RE, RING>(prob, c, g, sm);
   }
 }
 
