@@ -27,9 +27,18 @@ struct DenseProblem {
     h.Vf = sm.vf;
     h.Vd = sm.vd;
     h.Vx = sm.vx;
+    h.Ax = reinterpret_cast<cx<df>*>(sm.acc);
     return h;
   }
 };
+
+// The double-float kernels' matrix [A | b] or [A | I] in shared memory
+// (gj_solve_df), rows of one replica's lanes.
+template <int N, int PREC>
+__host__ __device__ constexpr int dense_acc_bytes() {
+  return PREC == HC_PREC_DF ? 16 * (2 * N) * ((N <= 4) ? 4 : (N <= 8) ? 8 : (N <= 16) ? 16 : 32)
+                            : 0;
+}
 
 // Resident blocks per SM the FP32 and FP64 kernels are compiled for (128
 // registers a thread); 3 and 5 (168 and 96 registers) measured no faster on
@@ -49,7 +58,7 @@ __global__ void __launch_bounds__(kBlock, PREC == HC_PREC_DF ? 1 : kTrackMinBloc
   using RE = typename std::conditional<XDF, df, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   const Group g = make_group<L, groups_meet(L, RING)>();
-  const GroupMem sm = make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, 0,
+  const GroupMem sm = make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(),
                                         endgame_smem_bytes(L, MIXED), XDF ? 1 : 0);
   DenseProblem<N, DEG, L> prob{&a, sm, g.meet};
   run_tracker<N, L, MIXED, DenseProblem<N, DEG, L>, RE, RING>(prob, a.c, g, sm);
@@ -61,7 +70,8 @@ template <int DEG, int PREC, int N, int LANES = 0, bool RING = false>
 KernelRef dense_ref() {
   constexpr int L = LANES ? LANES : ((N <= 4) ? 4 : (N <= 8) ? 8 : (N <= 16) ? 16 : 32);
   return KernelRef{reinterpret_cast<const void*>(&dense_td_kernel<N, DEG, PREC, L, RING>), L,
-                   DenseShape<N, DEG>::EXTRA, 0, endgame_smem_bytes(L, PREC == HC_PREC_MIXED),
+                   DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(),
+                   endgame_smem_bytes(L, PREC == HC_PREC_MIXED),
                    PREC == HC_PREC_DF ? 1 : 0};
 }
 

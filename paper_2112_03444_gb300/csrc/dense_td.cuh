@@ -27,7 +27,7 @@
 //      kernels.cuh); slice N pair 0 holds the constant c_i0.
 //   E: [M][L] complex double, nested Horner order; Edf the same entries as
 //      double-floats (16 bytes each: hi re, hi im, lo re, lo im).
-//   Ddf: D as complex double-floats (cx<df>: re hi, re lo, im hi, im lo), the
+//   Ddf: D as complex double-floats (cx<df>: re hi, im hi, re lo, im lo), the
 //      table of the double-float kernels, which evaluate with R = df.
 #pragma once
 
@@ -75,6 +75,7 @@ struct DenseTD {
   cx<float>* Vf;   // the group's shared copies of the evaluation point (+ monomials)
   cx<double>* Vd;
   cx<df>* Vx;      // double-float kernels: the point as double-floats (+ monomials)
+  cx<df>* Ax;      // and the row, entry j of row r at Ax[j * ROWL + r] (eval_rows)
   unsigned gmask;  // lanes that evaluate together (Group meet)
 
   template <class R>
@@ -83,8 +84,6 @@ struct DenseTD {
   __device__ __forceinline__ cx<R>* vptr() const {
     if constexpr (std::is_same<R, float>::value)
       return Vf;
-    else if constexpr (std::is_same<R, df>::value)
-      return Vx;
     else
       return Vd;
   }
@@ -97,6 +96,7 @@ struct DenseTD {
   // or 32 active lanes).
   static constexpr int PARTS = (L_GROUP > L) ? L_GROUP / L : 1;
   static constexpr int ROWL = (PARTS > 1) ? L : L_GROUP;  // lanes per row replica
+  static constexpr int WARPS = 1;
   static_assert(PARTS == 1 || L_GROUP == 32, "split rows need the whole warp");
 
   template <class R>
@@ -105,8 +105,7 @@ struct DenseTD {
 #pragma unroll
       for (int o = L; o < L * PARTS; o <<= 1) {
         if constexpr (std::is_same<R, df>::value) {
-          v.re = v.re + shfl_xor_df(v.re, o);
-          v.im = v.im + shfl_xor_df(v.im, o);
+          v = v + shfl_xor_df(v, o);
         } else {
           v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
           v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
@@ -161,6 +160,109 @@ struct DenseTD {
   template <class R>
   __device__ __forceinline__ void eval(const cx<R> (&)[N], int i, R t, R omt, cx<R> (&row)[N + 1],
                                        cx<R>& H, cx<R>& Ht) const {
+    if constexpr (std::is_same<R, df>::value) {
+      eval_rows(i, t, omt, H, Ht, WANT_HT | WANT_H);
+#pragma unroll
+      for (int j = 0; j < N; ++j) row[j] = Ax[j * ROWL + (i & (ROWL - 1))];
+    } else {
+      eval_row<R>(i, t, omt, row, H, Ht);
+    }
+  }
+
+  // The double-float form (split rows): the row goes to the group's shared
+  // memory, where gj_solve_df takes it, and every loop is rolled, one body of a
+  // multiply-add each: code size bounds these kernels (see run_tracker).  A
+  // lane takes JB slices at a time over its share of the monomials, two
+  // independent chains of multiply-adds.
+  enum : int { WANT_HT = 1, WANT_H = 2 };
+  __device__ __forceinline__ void eval_rows(int i, df t, df omt, cx<df>& H, cx<df>& Ht,
+                                            int) const {
+    constexpr int JB = 2;
+    const int r = i & (L - 1);
+    const int rr = r < N ? r : 0;
+    const int part = (PARTS > 1) ? i / L : 0;
+    auto pair = [&](int j, int q) {
+      return Ddf + ((int64_t)(j * (S::MPP / 2) + q) * L + rr) * 2;
+    };
+    cx<df>* V = Vx;
+    cx<df>* Q = V + L_GROUP;
+    if (i < N) V[i] = to_cxdf(Vd[i]);
+    __syncwarp(gmask);
+    if constexpr (DEG == 3) {
+#pragma unroll 1
+      for (int k = 0; k < N; ++k)
+        if (i < N - k) Q[S::idx2(k, k + i) - 1 - N] = V[k] * V[k + i];
+      __syncwarp(gmask);
+    }
+    // sums over this lane's share of the `count` monomial pairs at M (table
+    // pairs from `at`), for the slices j .. j + JB - 1
+    auto contract = [&](int j, const cx<df>* M, int at, int count, cx<df> (&acc)[JB]) {
+#pragma unroll
+      for (int b = 0; b < JB; ++b) acc[b] = czero<df>();
+#pragma unroll 1
+      for (int q = part; q < count; q += PARTS) {
+        const cx<df> m0 = M[2 * q], m1 = M[2 * q + 1];
+#pragma unroll
+        for (int b = 0; b < JB; ++b) {
+          const cx<df>* c = pair(min(j + b, N - 1), at + q);
+          acc[b] = cfma(c[1], m1, cfma(c[0], m0, acc[b]));
+        }
+      }
+    };
+    cx<df> fp = czero<df>();
+#pragma unroll 1
+    for (int j = 0; j < N; j += JB) {
+      cx<df> a1[JB], a2[JB];
+      contract(j, V, 1, S::N2 / 2, a1);
+      if constexpr (DEG == 3) contract(j, Q, 1 + S::N2 / 2, S::NQ2 / 2, a2);
+#pragma unroll
+      for (int b = 0; b < JB; ++b) {
+        if (j + b < N) {
+          if constexpr (DEG == 3) {
+            fp = cfma(V[j + b], df(0.5) * a1[b] + df(1.0 / 3.0) * a2[b], fp);
+            a1[b] = a1[b] + a2[b];
+          }
+          const cx<df> sum = part_sum(a1[b]);
+          if (part == 0) Ax[(j + b) * L + r] = sum;
+        }
+      }
+    }
+    __syncwarp(gmask);
+    cx<df> F = pair(N, 0)[0];
+    if constexpr (DEG == 3) F = F + part_sum(fp);
+#pragma unroll 1
+    for (int j = 0; j < N; ++j) {
+      const cx<df> a0 = pair(j, 0)[0];
+      F = cfma(V[j], DEG == 3 ? a0 : a0 + df(0.5) * Ax[j * L + r], F);
+    }
+    const cx<df> xi = V[rr];
+    const cx<df> xi2 = xi * xi;
+    const cx<df> G = (DEG == 2 ? xi2 : xi2 * xi) - mk<df>(df(1), df(0));
+    const cx<df> Gd = df(DEG) * (DEG == 2 ? xi : xi2);
+    const cx<df> gm = to_cxdf(gammadf);
+    const cx<df> gG = gm * G;
+    H = t * F + omt * gG;
+    Ht = F - gG;
+    const cx<df> gd = omt * (gm * Gd);
+    __syncwarp(gmask);  // every part has read the sums
+#pragma unroll 1
+    for (int j = part; j < N; j += PARTS) {
+      cx<df> v = t * (pair(j, 0)[0] + Ax[j * L + r]);
+      if (j == r) v = v + gd;
+      Ax[j * L + r] = v;
+    }
+    __syncwarp(gmask);
+  }
+
+  template <bool MEET>
+  __device__ __forceinline__ bool solve(const Group& g, cx<df>* A, cx<df>* pv, int W,
+                                        cx<df>& dinv, int& col) const {
+    return gj_solve_df<N, ROWL, PARTS, MEET>(g, A, pv, W, dinv, col);
+  }
+
+  template <class R>
+  __device__ __forceinline__ void eval_row(int i, R t, R omt, cx<R> (&row)[N + 1], cx<R>& H,
+                                           cx<R>& Ht) const {
     const int r = i & (L - 1);                   // this lane's row
     const int rr = r < N ? r : 0;
     const int part = (PARTS > 1) ? i / L : 0;    // and its share of the contraction
@@ -169,11 +271,6 @@ struct DenseTD {
     auto pair = [&](int j, int q) { return D + ((int64_t)(j * (S::MPP / 2) + q) * L + rr) * 2; };
     cx<R>* V = vptr<R>();
     cx<R>* Q = V + L_GROUP;
-    if constexpr (std::is_same<R, df>::value) {
-      // the tracker keeps the point in FP64 (Vd): split it once per evaluation
-      if (i < N) V[i] = to_cxdf(Vd[i]);
-      __syncwarp(gmask);
-    }
     if constexpr (DEG == 3) {
       // x_k x_l for k <= l in graded order: row k of the triangle, lane i
       // forming x_k x_(k+i) (no index search, no divergence)
@@ -255,8 +352,6 @@ struct DenseTD {
     cx<R> gm;
     if constexpr (std::is_same<R, float>::value)
       gm = gamma32;
-    else if constexpr (std::is_same<R, df>::value)
-      gm = to_cxdf(gammadf);
     else
       gm = gamma;
     const cx<R> gG = gm * G;
@@ -597,8 +692,6 @@ template <class R>
 __device__ __forceinline__ const cx<R>* DenseTD<N, DEG, LG>::dptr() const {
   if constexpr (std::is_same<R, float>::value)
     return D32;
-  else if constexpr (std::is_same<R, df>::value)
-    return Ddf;
   else
     return D64;
 }

@@ -96,13 +96,99 @@ __device__ __forceinline__ df df_add(df a, df b) {
   return r;
 }
 
-// Complex double-float: one 16-byte word (hi.re, hi.im, lo.re, lo.im) in
-// shared or global memory.
+// Packed form: the real and the imaginary part of a complex double-float run
+// the same operations, so each operation is one two-wide FP32 instruction
+// (FADD2, FMUL2, FFMA2) over (re, im).  These round each half as the scalar
+// instruction does -- the results are the scalar form's bit for bit -- and take
+// the FP32 pipe as long as two scalar ones (measured: 2 cycles a warp
+// instruction and scheduler, latency 5, negated operands free), but half the
+// issue slots and half the code: a complex multiply-add 97 -> 70 cycles with
+// one warp per scheduler and 73 -> 64 with four, and code is what the
+// double-float kernels stall on (see run_tracker).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = add2(a, b);
+  const float2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
+// Complex double-float in registers, shared and global memory: one 16-byte
+// word, high parts (re, im) then low parts.
+template <>
+struct __align__(16) cx<df> {
+  float2 h, l;
+};
+__device__ __forceinline__ df re_of(cx<df> z) { return df{z.h.x, z.l.x}; }
+__device__ __forceinline__ df im_of(cx<df> z) { return df{z.h.y, z.l.y}; }
+template <>
+__device__ __forceinline__ cx<df> mk<df>(df re, df im) {
+  return cx<df>{make_float2(re.hi, im.hi), make_float2(re.lo, im.lo)};
+}
+template <>
+__device__ __forceinline__ cx<df> czero<df>() {
+  return cx<df>{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+}
+
+// c + x1 y1 + x2 y2 in both halves (df_dot2)
+__device__ __forceinline__ cx<df> dot2p(cx<df> c, cx<df> x1, cx<df> y1, cx<df> x2, cx<df> y2) {
+  const float2 p1 = mul2(x1.h, y1.h), e1 = fma2(x1.h, y1.h, neg2(p1));
+  const float2 p2 = mul2(x2.h, y2.h), e2 = fma2(x2.h, y2.h, neg2(p2));
+  float2 l = fma2(x1.h, y1.l, fma2(x1.l, y1.h, e1));
+  l = add2(l, fma2(x2.h, y2.l, fma2(x2.l, y2.h, e2)));
+  float2 s, es, s2, es2;
+  two_sum2(c.h, p1, s, es);
+  two_sum2(s, p2, s2, es2);
+  const float2 lo = add2(add2(c.l, l), add2(es, es2));
+  cx<df> r;
+  two_sum2(s2, lo, r.h, r.l);
+  return r;
+}
+// x1 y1 + x2 y2 in both halves (df_sdot2)
+__device__ __forceinline__ cx<df> sdot2p(cx<df> x1, cx<df> y1, cx<df> x2, cx<df> y2) {
+  const float2 p1 = mul2(x1.h, y1.h), e1 = fma2(x1.h, y1.h, neg2(p1));
+  const float2 p2 = mul2(x2.h, y2.h), e2 = fma2(x2.h, y2.h, neg2(p2));
+  float2 l = fma2(x1.h, y1.l, fma2(x1.l, y1.h, e1));
+  l = add2(l, fma2(x2.h, y2.l, fma2(x2.l, y2.h, e2)));
+  float2 s, es;
+  two_sum2(p1, p2, s, es);
+  cx<df> r;
+  two_sum2(s, add2(l, es), r.h, r.l);
+  return r;
+}
+// x y in both halves (operator* of df)
+__device__ __forceinline__ cx<df> mulp(cx<df> x, cx<df> y) {
+  const float2 p = mul2(x.h, y.h);
+  const float2 e = fma2(x.h, y.l, fma2(x.l, y.h, fma2(x.h, y.h, neg2(p))));
+  cx<df> r;
+  two_sum2(p, e, r.h, r.l);
+  return r;
+}
+// operands of a complex product a b = (a.re b.re - a.im b.im,
+// a.re b.im + a.im b.re): both halves a.re; (-a.im, a.im); b swapped
+__device__ __forceinline__ cx<df> re_re(cx<df> a) { return {dup2(a.h.x), dup2(a.l.x)}; }
+__device__ __forceinline__ cx<df> nim_im(cx<df> a) {
+  return {make_float2(-a.h.y, a.h.y), make_float2(-a.l.y, a.l.y)};
+}
+__device__ __forceinline__ cx<df> im_re(cx<df> b) { return {swap2(b.h), swap2(b.l)}; }
+__device__ __forceinline__ cx<df> neg(cx<df> a) { return {neg2(a.h), neg2(a.l)}; }
+
+// The complex double-float of the residuals (tables, the mixed kernels' point
+// copies): the same word.
 struct __align__(16) cdf {
   float hr, hi_, lr, li;  // hi part (re, im), lo part (re, im)
-  __device__ __forceinline__ df re() const { return df{hr, lr}; }
-  __device__ __forceinline__ df im() const { return df{hi_, li}; }
+  __host__ __device__ df re() const { return df{hr, lr}; }
+  __host__ __device__ df im() const { return df{hi_, li}; }
 };
+__device__ __forceinline__ cx<df> to_cxdf(cdf z) {
+  return {make_float2(z.hr, z.hi_), make_float2(z.lr, z.li)};
+}
+__device__ __forceinline__ cdf to_cdf(cx<df> z) { return cdf{z.h.x, z.h.y, z.l.x, z.l.y}; }
 
 __device__ __forceinline__ cdf mk_cdf(df re, df im) { return cdf{re.hi, im.hi, re.lo, im.lo}; }
 __device__ __forceinline__ cdf to_cdf(cx<double> z) { return mk_cdf(to_df(z.re), to_df(z.im)); }
@@ -116,21 +202,26 @@ __device__ __forceinline__ cx<double> cdf_to_cd(cdf z) {
 
 // acc + a b
 __device__ __forceinline__ cdf cdf_fma(cdf a, cdf b, cdf acc) {
-  return mk_cdf(df_dot2(acc.re(), a.re(), b.re(), df_neg(a.im()), b.im()),
-                df_dot2(acc.im(), a.re(), b.im(), a.im(), b.re()));
+  const cx<df> pa = to_cxdf(a), pb = to_cxdf(b);
+  return to_cdf(dot2p(to_cxdf(acc), re_re(pa), pb, nim_im(pa), im_re(pb)));
 }
 // a b
 __device__ __forceinline__ cdf cdf_mul(cdf a, cdf b) { return cdf_fma(a, b, cdf_zero()); }
-__device__ __forceinline__ cdf cdf_add(cdf a, cdf b) {
-  return mk_cdf(df_add(a.re(), b.re()), df_add(a.im(), b.im()));
+__device__ __forceinline__ cx<df> addp(cx<df> a, cx<df> b) {
+  float2 s, e;
+  two_sum2(a.h, b.h, s, e);
+  cx<df> r;
+  two_sum2(s, add2(e, add2(a.l, b.l)), r.h, r.l);
+  return r;
 }
+__device__ __forceinline__ cdf cdf_add(cdf a, cdf b) { return to_cdf(addp(to_cxdf(a), to_cxdf(b))); }
 __device__ __forceinline__ cdf cdf_sub(cdf a, cdf b) {
-  return mk_cdf(df_add(a.re(), df_neg(b.re())), df_add(a.im(), df_neg(b.im())));
+  return to_cdf(addp(to_cxdf(a), neg(to_cxdf(b))));
 }
 // a real double-float times a complex one
 __device__ __forceinline__ cdf cdf_scale(df s, cdf a) {
-  const df z{0.f, 0.f};
-  return mk_cdf(df_dot2(z, s, a.re(), z, z), df_dot2(z, s, a.im(), z, z));
+  const cx<df> z = czero<df>();
+  return to_cdf(dot2p(z, cx<df>{dup2(s.hi), dup2(s.lo)}, to_cxdf(a), z, z));
 }
 
 // host-side split of a complex double (tables and launch arguments)
@@ -185,34 +276,110 @@ __device__ __forceinline__ df df_recip(df d) {
 
 // Complex operations on cx<df> (overloads of the templates in
 // hc_device.cuh; a complex product is two two-term dot products).
+__device__ __forceinline__ cx<df> operator+(cx<df> a, cx<df> b) { return addp(a, b); }
+__device__ __forceinline__ cx<df> operator-(cx<df> a) { return neg(a); }
+__device__ __forceinline__ cx<df> operator-(cx<df> a, cx<df> b) { return addp(a, neg(b)); }
+__device__ __forceinline__ cx<df> operator*(df s, cx<df> a) {
+  return mulp(cx<df>{dup2(s.hi), dup2(s.lo)}, a);
+}
 __device__ __forceinline__ cx<df> operator*(cx<df> a, cx<df> b) {
-  return {df_sdot2(a.re, b.re, -a.im, b.im), df_sdot2(a.re, b.im, a.im, b.re)};
+  return sdot2p(re_re(a), b, nim_im(a), im_re(b));
 }
 __device__ __forceinline__ cx<df> cfma(cx<df> a, cx<df> b, cx<df> acc) {
-  return {df_dot2(acc.re, a.re, b.re, -a.im, b.im), df_dot2(acc.im, a.re, b.im, a.im, b.re)};
+  return dot2p(acc, re_re(a), b, nim_im(a), im_re(b));
 }
 __device__ __forceinline__ cx<df> cfms(cx<df> a, cx<df> b, cx<df> acc) {
-  return {df_dot2(acc.re, -a.re, b.re, a.im, b.im), df_dot2(acc.im, -a.re, b.im, -a.im, b.re)};
+  return dot2p(acc, neg(re_re(a)), b, neg(nim_im(a)), im_re(b));
 }
 // 1/z = conj(z) / |z|^2 (|z| must stay inside FP32's range, as for the
 // FP32 solve: a pivot outside it gives a non-finite reciprocal and the step
 // is rejected)
 __device__ __forceinline__ cx<df> crecip(cx<df> z) {
-  const df inv = df_recip(df_sdot2(z.re, z.re, z.im, z.im));
-  return {z.re * inv, -(z.im * inv)};
+  const df re = re_of(z), im = im_of(z);
+  const df inv = df_recip(df_sdot2(re, re, im, im));
+  const cx<df> r = mulp(z, cx<df>{dup2(inv.hi), dup2(inv.lo)});
+  return {make_float2(r.h.x, -r.h.y), make_float2(r.l.x, -r.l.y)};
 }
 // magnitudes for pivot choice and tests: FP32 accuracy from the high parts
-__device__ __forceinline__ float cabs1(cx<df> z) { return fabsf(z.re.hi) + fabsf(z.im.hi); }
-__device__ __forceinline__ float cnorm2(cx<df> z) {
-  return fmaf(z.re.hi, z.re.hi, z.im.hi * z.im.hi);
-}
+__device__ __forceinline__ float cabs1(cx<df> z) { return fabsf(z.h.x) + fabsf(z.h.y); }
+__device__ __forceinline__ float cnorm2(cx<df> z) { return fmaf(z.h.x, z.h.x, z.h.y * z.h.y); }
 __device__ __forceinline__ float cabs2(cx<df> z) { return sqrtf(cnorm2(z)); }
 // complex double <-> complex double-float
-__device__ __forceinline__ cx<df> to_cxdf(cx<double> z) { return {df(z.re), df(z.im)}; }
-__device__ __forceinline__ cx<df> to_cxdf(cdf z) { return {z.re(), z.im()}; }
+__device__ __forceinline__ cx<df> to_cxdf(cx<double> z) { return mk<df>(df(z.re), df(z.im)); }
 // butterfly sum over the lanes xor o (o = L .. L * PARTS / 2) of a warp
 __device__ __forceinline__ df shfl_xor_df(df v, int o) {
   return df{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ cx<df> shfl_xor_df(cx<df> v, int o) {
+  return {make_float2(__shfl_xor_sync(0xffffffffu, v.h.x, o),
+                      __shfl_xor_sync(0xffffffffu, v.h.y, o)),
+          make_float2(__shfl_xor_sync(0xffffffffu, v.l.x, o),
+                      __shfl_xor_sync(0xffffffffu, v.l.y, o))};
+}
+
+// The elimination of gj_solve (hc_device.cuh) for double-float rows held in
+// shared memory: entry j of row r at A[j * LR + r], LR = lanes per row replica,
+// PARTS replicas (lane gl: row gl mod LR, columns j with j mod PARTS = gl / LR).
+// Rolled over the pivots and over the columns (UNROLL of a lane's columns at a
+// time, to cover the chain of a multiply-add): unrolled with the row in
+// registers, the solve alone was 60 to 150 KB of code, and a path's warp,
+// often the only one of its scheduler, waited for instructions at 5.6 cycles
+// each (see run_tracker).  Measured with the packed arithmetic and rolled
+// evaluations, ms: precision DF on cubic n = 8 (16 systems) 3464 -> 430, on quadratic
+// n = 6 (64) 27.7 -> 7.4; re-tracking of cubic n = 8 31.5 -> 18.9.  The same
+// operations in the same order per entry, so the same results.  W columns: N and the right-hand sides.  pv: W entries.  On
+// return the lanes of part 0 hold in col the column they pivoted on (-1: none)
+// and in dinv 1 / pivot: that component of x is dinv times the right-hand side.
+template <int N, int LR, int PARTS, bool MEET>
+__device__ __forceinline__ bool gj_solve_df(const Group& g, cx<df>* A, cx<df>* pv, int W,
+                                            cx<df>& dinv, int& col) {
+  constexpr int L = LR * PARTS;
+  constexpr int UNROLL = PARTS >= 4 ? 2 : 3;
+  const int r = g.gl & (LR - 1), part = PARTS > 1 ? g.gl / LR : 0;
+  bool used = r >= N;
+  dinv = mk<df>(df(1), df(0));
+  unsigned lo = 0xffffffffu, hi = 0u;
+  col = -1;
+#pragma unroll 1
+  for (int k = 0; k < N; ++k) {
+    const cx<df> ak = A[k * LR + r];
+    const float m = cabs1(ak);
+    const unsigned key = used ? 0u : ((__float_as_uint(m) & ~31u) | (unsigned)(31 - r));
+    const unsigned kmax = gmaxu<L, MEET>(g, key);
+    const cx<df> inv = crecip(ak);
+    lo = min(lo, kmax);
+    hi = max(hi, kmax);
+    const int rp = min(31 - (int)(kmax & 31u), LR - 1);  // the pivot row
+    const bool me = r == rp;
+    for (int j = k + 1 + g.gl; j < W; j += L) pv[j] = A[j * LR + rp];
+    if (me) {
+      if (part == 0) pv[k] = inv;
+      used = true;
+      dinv = inv;
+      col = k;
+    }
+    __syncwarp(g.meet);
+    const cx<df> l = me ? czero<df>() : ak * pv[k];
+    const cx<df> lr = neg(re_re(l)), li = neg(nim_im(l));
+    // a lane's first column behind k
+    const int j0 = k + 1 + (PARTS > 1 ? ((part - (k + 1)) & (PARTS - 1)) : 0);
+#pragma unroll 1
+    for (int j = j0; j < W; j += UNROLL * PARTS) {
+      cx<df> a[UNROLL];
+#pragma unroll
+      for (int u = 0; u < UNROLL; ++u) {
+        const int ju = min(j + u * PARTS, W - 1);
+        const cx<df> p = pv[ju];
+        a[u] = dot2p(A[ju * LR + r], lr, p, li, im_re(p));
+      }
+#pragma unroll
+      for (int u = 0; u < UNROLL; ++u)
+        if (j + u * PARTS < W) A[(j + u * PARTS) * LR + r] = a[u];
+    }
+    __syncwarp(g.meet);
+  }
+  if (part != 0 || r >= N) col = -1;
+  return (lo & ~31u) != 0u && (hi & ~31u) < 0x7f800000u;
 }
 
 }  // namespace hc

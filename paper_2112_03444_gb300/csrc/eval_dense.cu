@@ -16,7 +16,8 @@ __global__ void __launch_bounds__(kBlock) dense_eval(const DenseEvalArgs ea) {
   extern __shared__ __align__(16) unsigned char smem[];
   const Group g = make_group<L>();
   const GroupMem sm =
-      make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, 0, 0, PREC == HC_PREC_DF ? 1 : 0);
+      make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(), 0,
+                        PREC == HC_PREC_DF ? 1 : 0);
   DenseProblem<N, DEG, L> prob{&ea.a, sm, g.mask};
   eval_points<N, L, R>(prob, ea.e, g, sm);
 }
@@ -25,7 +26,8 @@ template <int DEG, int PREC, int N>
 KernelRef dense_eval_ref() {
   constexpr int L = PREC == HC_PREC_DF ? 32 : ((N <= 4) ? 4 : (N <= 8) ? 8 : 16);
   return KernelRef{reinterpret_cast<const void*>(&dense_eval<N, DEG, PREC, L>), L,
-                   DenseShape<N, DEG>::EXTRA, 0, 0, PREC == HC_PREC_DF ? 1 : 0};
+                   DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(), 0,
+                   PREC == HC_PREC_DF ? 1 : 0};
 }
 
 template <int DEG, int PREC, int N>

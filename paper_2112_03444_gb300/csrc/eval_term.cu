@@ -5,6 +5,7 @@
 #include <type_traits>
 
 #include "evaluate.cuh"
+#include "term_block.cuh"
 #include "term_param.cuh"
 
 namespace hc {
@@ -12,22 +13,32 @@ namespace hc {
 template <int N, int PREC, int L>
 __global__ void __launch_bounds__(kBlock) term_eval(const __grid_constant__ TermEvalArgs ea) {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
-  using R = typename std::conditional<
-      MIXED, float, typename std::conditional<PREC == HC_PREC_DF, df, double>::type>::type;
+  using R = typename std::conditional<MIXED, float, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   const Group g = make_group<L>();
-  const GroupMem sm = make_group_mem<L>(smem, ea.a.extra, term_acc_bytes<N, MIXED, L>(), 0,
-                                        PREC == HC_PREC_DF ? 1 : 0);
+  const GroupMem sm = make_group_mem<L>(smem, ea.a.extra, term_acc_bytes<N, MIXED, L>());
   TermProblem<N, L, MIXED> prob{&ea.a, g, sm};
   eval_points<N, L, R>(prob, ea.e, g, sm);
 }
 
+template <int N>
+__global__ void __launch_bounds__(kBlock) term_eval_df(const __grid_constant__ TermEvalArgs ea) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Group g = make_group<32>();
+  const GroupMem sm =
+      make_group_mem<32>(smem, ea.a.extra, TermBlock<N, 1>::acc_bytes(), 0, 1);
+  TermBlockProblem<N, 1> prob{&ea.a, g, sm};
+  eval_points<N, 32, df>(prob, ea.e, g, sm);
+}
+
 template <int PREC, int N>
 KernelRef term_eval_ref() {
+  if constexpr (PREC == HC_PREC_DF)
+    return KernelRef{reinterpret_cast<const void*>(&term_eval_df<N>), 32, 0,
+                     TermBlock<N, 1>::acc_bytes(), 0, 1};
   constexpr int L = (N <= 4) ? 4 : (N <= 8) ? 8 : (N <= 16) ? 16 : 32;
   return KernelRef{reinterpret_cast<const void*>(&term_eval<N, PREC, L>), L, 0,
-                   term_acc_bytes<N, PREC == HC_PREC_MIXED, L>(), 0,
-                   PREC == HC_PREC_DF ? 1 : 0};
+                   term_acc_bytes<N, PREC == HC_PREC_MIXED, L>(), 0, 0};
 }
 
 template <int PREC, int N>

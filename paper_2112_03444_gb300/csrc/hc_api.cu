@@ -31,12 +31,12 @@ KernelRef dense_ref_d3_df(int n);
 
 KernelRef term_ref_64(int n, int lanes);
 KernelRef term_ref_32(int n, int lanes);
-KernelRef term_ref_df(int n);
+KernelRef term_ref_df(int n, int lanes);
 
-// The double-float kernels come in one width each: one path per warp for
-// dense systems, the default width for term tables.
+// The double-float kernels: one path per warp for dense systems; for term
+// tables one or more warps per path (lanes = 32: one).
 KernelRef term_kernel(int n, int prec, int lanes) {
-  if (prec == HC_PREC_DF) return term_ref_df(n);
+  if (prec == HC_PREC_DF) return term_ref_df(n, lanes);
   return prec == HC_PREC_MIXED ? term_ref_32(n, lanes) : term_ref_64(n, lanes);
 }
 
@@ -97,9 +97,9 @@ __global__ void stage_dense_kernel(int64_t n_inst, int T, const double2* __restr
       const double2 dv = make_double2(m * v.x, m * v.y);
       if (D64) D64[inst * Ds + dslot[r]] = dv;
       if (D32) D32[inst * Ds + dslot[r]] = make_float2((float)dv.x, (float)dv.y);
-      if (Ddf) {  // cx<df> layout: re hi, re lo, im hi, im lo
+      if (Ddf) {  // cx<df> layout: re hi, im hi, re lo, im lo
         const hc::df re(dv.x), im(dv.y);
-        Ddf[inst * Ds + dslot[r]] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        Ddf[inst * Ds + dslot[r]] = make_float4(re.hi, im.hi, re.lo, im.lo);
       }
     }
   }
@@ -927,7 +927,7 @@ hc_status launch_generic(const hc::KernelRef& k, void* args, size_t smem, int64_
   if (smem > 48 * 1024)
     HC_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const Occ o = occupancy(k.fn, smem, threads);
-  const int64_t groups_per_block = threads / k.lanes;
+  const int64_t groups_per_block = threads / (k.lanes * k.warps);
   int64_t want = (max_items + groups_per_block - 1) / groups_per_block;
   int64_t grid = std::min<int64_t>((int64_t)o.blocks * o.sms, std::max<int64_t>(want, 1));
   void* argv[] = {args};
@@ -938,7 +938,7 @@ hc_status launch_generic(const hc::KernelRef& k, void* args, size_t smem, int64_
 hc_status launch_tracker(const hc::KernelRef& k, const hc::DenseArgs& a, int64_t max_items,
                          cudaStream_t st, int threads = hc::kBlock) {
   const size_t smem =
-      (size_t)hc::block_smem_bytes(k.lanes, k.extra, 0, threads, k.eg_bytes, k.vx);
+      (size_t)hc::block_smem_bytes(k.lanes, k.extra, k.acc_bytes, threads, k.eg_bytes, k.vx);
   return launch_generic(k, (void*)&a, smem, max_items, st, threads);
 }
 
@@ -1545,12 +1545,13 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
     const hc::KernelRef k = hc::term_kernel(n, p->s.precision, mixed ? p->s.lanes : 0);
     auto smem_of = [&](const hc::KernelRef& kr, int threads = hc::kBlock) {
       return (size_t)hc::block_smem_bytes(kr.lanes, p->extra, kr.acc_bytes, threads, kr.eg_bytes,
-                                          kr.vx);
+                                          kr.vx, kr.warps);
     };
     // fewer paths per block where a block's groups would not fit in shared
     // memory (many parameters: V holds 1 + 3 P entries per group)
     const size_t smem_cap = max_block_smem();
     auto fit = [&](const hc::KernelRef& kr, int threads) {
+      if (kr.warps > 1) return hc::block_threads(kr.warps, threads);
       while (threads > 32 && threads > kr.lanes && smem_of(kr, threads) > smem_cap) threads /= 2;
       return threads;
     };
@@ -2518,7 +2519,7 @@ extern "C" hc_status hc_evaluate(const hc_problem* p, int32_t precision, int32_t
       a.gamma32 = cx<float>{(float)p->gamma[0], (float)p->gamma[1]};
       a.gammadf = hc::split_cdf_host(p->gamma[0], p->gamma[1]);
       da.e = e;
-      smem = (size_t)hc::block_smem_bytes(k.lanes, k.extra, 0, threads, 0, k.vx);
+      smem = (size_t)hc::block_smem_bytes(k.lanes, k.extra, k.acc_bytes, threads, 0, k.vx);
       argp = &da;
     }
     if (smem > 48 * 1024)
@@ -2654,7 +2655,8 @@ extern "C" hc_status hc_stream_create(hc_problem* p, int32_t slots, int64_t idle
   s->kt = hc::ring_kernel(p->terms, p->deg, n);
   if (p->terms) {
     s->kr = hc::term_kernel(n, HC_PREC_MIXED, 0);
-    s->kl = hc::term_kernel(n, hc::last_tier_precision(p->s), 0);
+    const int last = hc::last_tier_precision(p->s);
+    s->kl = hc::term_kernel(n, last, last == HC_PREC_DF ? 32 : 0);
   } else {
     s->kr = retrack_kernel(p->deg, n, HC_PREC_MIXED);
     s->kl = retrack_kernel(p->deg, n, hc::last_tier_precision(p->s));
@@ -2744,7 +2746,7 @@ extern "C" hc_status hc_stream_create(hc_problem* p, int32_t slots, int64_t idle
   s->threads = std::max(main_threads(p->s), s->kt.lanes);
   s->smem = p->terms ? (size_t)hc::block_smem_bytes(s->kt.lanes, p->extra, s->kt.acc_bytes,
                                                      s->threads, s->kt.eg_bytes, s->kt.vx)
-                     : (size_t)hc::block_smem_bytes(s->kt.lanes, s->kt.extra, 0, s->threads,
+                     : (size_t)hc::block_smem_bytes(s->kt.lanes, s->kt.extra, s->kt.acc_bytes, s->threads,
                                                     s->kt.eg_bytes, s->kt.vx);
   if (s->smem > 48 * 1024 &&
       cudaFuncSetAttribute(s->kt.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,

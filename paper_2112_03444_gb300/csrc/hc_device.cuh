@@ -87,8 +87,12 @@ __device__ __forceinline__ R cabs1(cx<R> z) { return fabs(z.re) + fabs(z.im); }
 template <class R>
 __device__ __forceinline__ R cabs2(cx<R> z) { return sqrt(fma(z.re, z.re, z.im * z.im)); }
 
+template <class R>
+__device__ __forceinline__ R re_of(cx<R> z) { return z.re; }
+template <class R>
+__device__ __forceinline__ R im_of(cx<R> z) { return z.im; }
 template <class D, class S>
-__device__ __forceinline__ cx<D> cvt(cx<S> z) { return {(D)z.re, (D)z.im}; }
+__device__ __forceinline__ cx<D> cvt(cx<S> z) { return mk<D>((D)re_of(z), (D)im_of(z)); }
 
 template <class R>
 __device__ __forceinline__ bool cfinite(cx<R> z) { return isfinite(z.re) && isfinite(z.im); }

@@ -32,14 +32,17 @@ __host__ __device__ constexpr int group_smem_bytes(int L, int extra, int acc = 0
 __host__ __device__ constexpr int endgame_smem_bytes(int L, bool mixed) { return mixed ? 0 : 48 * L; }
 // Dynamic shared memory of one tracking block of `threads` threads
 __host__ __device__ constexpr int block_smem_bytes(int L, int extra, int acc = 0,
-                                                   int threads = kBlock, int eg = 0, int vx = 0) {
-  return (threads / L) * group_smem_bytes(L, extra, acc, eg, vx);
+                                                   int threads = kBlock, int eg = 0, int vx = 0,
+                                                   int warps = 1) {
+  return (threads / (L * warps)) * group_smem_bytes(L, extra, acc, eg, vx);
 }
 // Threads per block of a launch: one warp for one-path-per-warp launches of
 // the re-tracking tiers (a hard path then holds only its own warp's
 // registers, not three idle warps' beside the other classes' launches),
 // kBlock otherwise.
 inline int retrack_threads(int lanes) { return lanes == 32 ? 32 : kBlock; }
+// A kernel with several warps per path takes blocks of exactly one path.
+inline int block_threads(int warps, int want) { return warps > 1 ? 32 * warps : want; }
 
 // Dense coefficient tables D (see dense_td.cuh): per slice j (the partial
 // derivative dF_i/dx_j; slice n holds the constant term), the monomials of
@@ -202,6 +205,7 @@ struct KernelRef {
   int acc_bytes;    // bytes of one evaluator accumulator (per lane and row entry), 0: none
   int eg_bytes;     // per-group endgame sample bytes (FP64-state kernels), 0: none
   int vx;           // 1: double-float kernel (a double-float copy of the point)
+  int warps = 1;    // warps per path (lanes = 32)
 };
 
 // Lanes per path chosen for n unknowns (one row per lane, groups are powers

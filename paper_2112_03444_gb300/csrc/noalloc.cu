@@ -136,9 +136,9 @@ __device__ __forceinline__ void put_d(double2* D64, float2* D32, float4* Ddf, in
                                       double2 v) {
   D64[slot] = v;
   D32[slot] = make_float2((float)v.x, (float)v.y);
-  if (Ddf) {  // cx<df> layout: re hi, re lo, im hi, im lo
+  if (Ddf) {  // cx<df> layout: re hi, im hi, re lo, im lo
     const hc::df re(v.x), im(v.y);
-    Ddf[slot] = make_float4(re.hi, re.lo, im.hi, im.lo);
+    Ddf[slot] = make_float4(re.hi, im.hi, re.lo, im.lo);
   }
 }
 
@@ -325,7 +325,7 @@ extern "C" hc_status hc_track_dense_noalloc(int32_t n, int32_t degree, const dou
   auto launch = [&](const hc::KernelRef& k, const hc::DenseArgs& args, int64_t max_items,
                     int threads = hc::kBlock) {
     const size_t smem =
-        (size_t)hc::block_smem_bytes(k.lanes, k.extra, 0, threads, k.eg_bytes, k.vx);
+        (size_t)hc::block_smem_bytes(k.lanes, k.extra, k.acc_bytes, threads, k.eg_bytes, k.vx);
     int blocks = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k.fn, threads, smem) !=
         cudaSuccess)

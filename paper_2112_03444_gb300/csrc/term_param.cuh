@@ -40,11 +40,7 @@ namespace hc {
 // value first on both lanes so that the two copies agree bit for bit.
 template <class R>
 __device__ __forceinline__ R pair_sum(R v, int o, bool upper) {
-  R w;
-  if constexpr (std::is_same<R, df>::value)
-    w = shfl_xor_df(v, o);
-  else
-    w = __shfl_xor_sync(0xffffffffu, v, o);
+  const R w = __shfl_xor_sync(0xffffffffu, v, o);
   return upper ? w + v : v + w;
 }
 template <class R>
@@ -64,6 +60,7 @@ struct TermEval {
   // so that the warp's lanes all work.  Otherwise one row per lane.
   static constexpr int PARTS = (L == 32 && N <= 16) ? 2 : 1;
   static constexpr int ROWL = L / PARTS;
+  static constexpr int WARPS = 1;
   // residuals are computed by each group alone (no cooperative form)
   static constexpr bool kCoop = false;
   const TermArgs* a;
@@ -72,7 +69,6 @@ struct TermEval {
   cx<float>* Vf;
   cx<double>* Vd;
   unsigned char* acc;  // [N + 2][L] accumulators of cx<R>, this lane at column g.gl
-  cx<df>* Vx;          // double-float kernels: V as double-floats; nullptr otherwise
 
   // constant part of V for this path: the 1, dp and p0 (FP32 copies, and
   // for DF double-float copies of dp and p0 in Vd)
@@ -87,13 +83,8 @@ struct TermEval {
       else
         Vd[LS] = mk<double>(1.0, 0.0);
     }
-    if (Vx && g.gl == 0) Vx[LS] = mk<df>(df(1), df(0));
     for (int l = g.gl; l < P; l += L) {
       const cx<double> d = mk<double>(p1[l].x - a->p0[l].x, p1[l].y - a->p0[l].y);
-      if (Vx) {
-        Vx[LS + 1 + P + l] = to_cxdf(d);
-        Vx[LS + 1 + 2 * P + l] = to_cxdf(mk<double>(a->p0[l].x, a->p0[l].y));
-      }
       if constexpr (DF) {
         Vdf[LS + 1 + P + l] = to_cdf(d);
         Vdf[LS + 1 + 2 * P + l] = to_cdf(mk<double>(a->p0[l].x, a->p0[l].y));
@@ -114,25 +105,18 @@ struct TermEval {
   __device__ __forceinline__ cx<R>* vptr() const {
     if constexpr (std::is_same<R, float>::value)
       return Vf;
-    else if constexpr (std::is_same<R, df>::value)
-      return Vx;
     else
       return Vd;
   }
 
   // p(t) into V (each lane a share), then wait for `lanes`.  FP64:
-  // (1-t) p0 + t p1 from the inputs; FP32: p0 + t dp from the FP32 copies;
-  // double-float: p0 + t dp from the double-float copies, and the point
-  // (which the tracker keeps in FP64 in Vd) split into double-floats.
+  // (1-t) p0 + t p1 from the inputs; FP32: p0 + t dp from the FP32 copies.
   template <class R>
   __device__ __forceinline__ void put_params(R t, unsigned lanes) const {
     const int P = a->P, LS = a->ls;
     if constexpr (std::is_same<R, float>::value) {
       for (int l = g.gl; l < P; l += L)
         Vf[LS + 1 + l] = cfma(mk<float>(t, 0.f), Vf[LS + 1 + P + l], Vf[LS + 1 + 2 * P + l]);
-    } else if constexpr (std::is_same<R, df>::value) {
-      if (g.gl < N) Vx[g.gl] = to_cxdf(Vd[g.gl]);
-      for (int l = g.gl; l < P; l += L) Vx[LS + 1 + l] = Vx[LS + 1 + 2 * P + l] + t * Vx[LS + 1 + P + l];
     } else {
       const double2* p1 = a->p1 + inst * P;
       // DF: the 1 of V is held as a double-float between FP64 residuals
@@ -184,9 +168,6 @@ struct TermEval {
       const float2 c = a->c0f[r], d = a->dcf[rd];
       dcr = mk<float>(d.x, d.y);
       s = cfma(mk<float>(t, 0.f), dcr, mk<float>(c.x, c.y));
-    } else if constexpr (std::is_same<R, df>::value) {
-      dcr = to_cxdf(a->dcdf[rd]);
-      s = to_cxdf(a->c0df[r]) + t * dcr;
     } else {
       const double2 c = a->c0[r], d = a->dc[rd];
       dcr = mk<double>(d.x, d.y);
@@ -214,8 +195,6 @@ struct TermEval {
         coef_at<R>(r, t, s, dcr);
       else if constexpr (std::is_same<R, float>::value)
         s = mk<float>(rc.s.x, rc.s.y);
-      else if constexpr (std::is_same<R, df>::value)
-        s = to_cxdf(a->sdf[r]);
       else
         s = mk<double>(a->s64[r].x, a->s64[r].y);
       cx<R> run = czero<R>();
@@ -326,7 +305,7 @@ struct TermProblem {
   Group g;
   GroupMem sm;
   __device__ __forceinline__ TermEval<N, L, DF> hom(int64_t inst) const {
-    return TermEval<N, L, DF>{a, inst, g, sm.vf, sm.vd, sm.acc, sm.vx};
+    return TermEval<N, L, DF>{a, inst, g, sm.vf, sm.vd, sm.acc};
   }
 };
 
@@ -336,18 +315,16 @@ __host__ __device__ constexpr int term_acc_bytes() {
   return (N + 1) * L * (MIXED ? 8 : 16);
 }
 
-// PREC: HC_PREC_MIXED, HC_PREC_FP64 or HC_PREC_DF (as the dense kernels)
+// PREC: HC_PREC_MIXED or HC_PREC_FP64 (double-float: term_block.cuh)
 template <int N, int PREC, int L, bool RING = false>
 __global__ void __launch_bounds__(kBlock) term_param_kernel(const __grid_constant__ TermArgs a) {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
-  constexpr bool XDF = PREC == HC_PREC_DF;
-  using RE = typename std::conditional<XDF, df, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   const Group g = make_group<L, groups_meet(L, RING)>();
   const GroupMem sm = make_group_mem<L>(smem, a.extra, term_acc_bytes<N, MIXED, L>(),
-                                        endgame_smem_bytes(L, MIXED), XDF ? 1 : 0);
+                                        endgame_smem_bytes(L, MIXED));
   TermProblem<N, L, MIXED> prob{&a, g, sm};
-  run_tracker<N, L, MIXED, TermProblem<N, L, MIXED>, RE, RING>(prob, a.c, g, sm);
+  run_tracker<N, L, MIXED, TermProblem<N, L, MIXED>, double, RING>(prob, a.c, g, sm);
 }
 
 template <int PREC, int N, int LANES = 0, bool RING = false>
@@ -355,8 +332,7 @@ KernelRef term_ref() {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
   constexpr int L = LANES ? LANES : ((N <= 4) ? 4 : (N <= 8) ? 8 : (N <= 16) ? 16 : 32);
   return KernelRef{reinterpret_cast<const void*>(&term_param_kernel<N, PREC, L, RING>), L, 0,
-                   term_acc_bytes<N, MIXED, L>(), endgame_smem_bytes(L, MIXED),
-                   PREC == HC_PREC_DF ? 1 : 0};
+                   term_acc_bytes<N, MIXED, L>(), endgame_smem_bytes(L, MIXED), 0};
 }
 
 }  // namespace hc

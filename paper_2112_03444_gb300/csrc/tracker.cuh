@@ -22,7 +22,7 @@
 //
 // Precision tiers.
 //   MIXED = false, RE = double: every operation in complex FP64 (the plain form).
-//   MIXED = false, RE = df: the same state, time, step control, corrector
+//   MIXED = false, RE = df (rows in shared memory): the same state, time, step control, corrector
 //     and refinement residuals and classification in FP64, but the RK4
 //     stages, the Jacobians and the solves -- nearly all of the arithmetic --
 //     in complex double-float arithmetic (FP32 pairs, about 48 bits, see
@@ -74,12 +74,6 @@
 #include "kernels.cuh"
 
 namespace hc {
-
-template <int N, class S, class R>
-__device__ __forceinline__ void load_vec(const cx<S>* buf, cx<R> (&x)[N]) {
-#pragma unroll
-  for (int k = 0; k < N; ++k) x[k] = cvt<R>(buf[k]);
-}
 
 // M_IDLE: a group without work waiting for the other groups of its warp
 // (kernels with cooperative residuals, which keep the warp together)
@@ -165,9 +159,9 @@ struct GroupMem {
 template <int L>
 __device__ __forceinline__ GroupMem make_group_mem(unsigned char* smem, int extra,
                                                    int acc_bytes = 0, int eg_bytes = 0,
-                                                   int vx = 0) {
+                                                   int vx = 0, int warps = 1) {
   const int stride = group_smem_bytes(L, extra, acc_bytes, eg_bytes, vx);
-  unsigned char* b = smem + (threadIdx.x / L) * stride;
+  unsigned char* b = smem + (threadIdx.x / (L * warps)) * stride;
   GroupMem m;
   m.stride = stride;
   // the 16 bytes by which the stride passes a multiple of 128 are not used
@@ -264,6 +258,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
   // drift apart and each runs the evaluation and the solve on its own.
   constexpr bool MEET = groups_meet(L, RING);
   constexpr int EP = COOP_EVAL ? 32 / L : 1;
+  constexpr int GL = L * HOM::WARPS;  // threads of a path
   const DevSettings& s = c.s;
   cx<R>* sb = reinterpret_cast<cx<R>*>(sm.sb);
   const bool act = g.gl < N;
@@ -320,8 +315,6 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
   const bool eg_on = !MIXED && s.endgame != 0;
   auto eg_active = [&]() { return eg_on && eg_next < s.eg_samples; };
 
-  cx<R> row[N + 1];
-  cx<R> x[N];
   cx<R> sol[1];
   int col;
 
@@ -656,12 +649,12 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
       } else if (c.spread && first_fetch) {
         // ticket = slot * blocks + block: consecutive items on different blocks
         // (and so, for the first blocks of the grid, on different SMs)
-        q = (unsigned long long)(threadIdx.x / L) * gridDim.x + blockIdx.x;
+        q = (unsigned long long)(threadIdx.x / GL) * gridDim.x + blockIdx.x;
         first_fetch = false;
       } else {
         if (g.gl == 0) q = atomicAdd(c.queue, 1ull);
         q = __shfl_sync(g.mask, q, leader);
-        if (c.spread) q += (unsigned long long)gridDim.x * (blockDim.x / L);
+        if (c.spread) q += (unsigned long long)gridDim.x * (blockDim.x / GL);
       }
       if (!RING && !stop) stop = (int64_t)q >= total;
       if (stop) {
@@ -778,12 +771,6 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
       if (act) sm.vf[g.gl] = cvt<float>(xd);
     }
     __syncwarp(g.meet);
-    if constexpr (MIXED) {
-      load_vec<N, float, float>(sm.vf, x);
-    } else {
-      load_vec<N, double, R>(sm.vd, x);
-    }
-
     if constexpr (MEET) {
       const unsigned live = __ballot_sync(0xffffffffu, g.gl == 0 && mode != M_IDLE);
       if (live == 0u) break;
@@ -832,7 +819,76 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
     }
 
     // ---- 2. row i of [dH/dx | rhs] and the solve
-    {
+    // the right-hand side of a residual pass
+    auto residual_rhs = [&]() -> cx<R> {
+      if constexpr (COOP) {
+        const float4 v = reinterpret_cast<const float4*>(sm.sb)[g.gl];
+        return mk<R>(R(-v.x), R(-v.y));
+      } else if constexpr (MIXED) {
+        if (mode == M_REFINE || !res64) {
+          cx<float> Hf;
+          float sc;
+          hom.template residual_df<false, EP>(reinterpret_cast<const cdf*>(sm.vd), g.gl, te, Hf,
+                                              sc);
+          return cvt<R>(-Hf);
+        }
+      }
+      cx<double> H64;
+      double sc;
+      hom.template residual64<false, EP>(sm.vd, g.gl, te, 1.0 - te, H64, sc);
+      return cvt<R>(-H64);
+    };
+    bool sok;
+    if constexpr (XDF) {
+      // the row lives in shared memory (HOM::eval_rows, gj_solve_df)
+      cx<df>* A = reinterpret_cast<cx<df>*>(sm.acc);
+      const int grow = g.gl & (HOM::ROWL - 1);
+      cx<df> H, Ht, dinv;
+      cx<df>* pv = reinterpret_cast<cx<df>*>(sm.pv);
+      // RK stages take dH/dt, Newton steps H (unless it comes from a residual)
+      hom.eval_rows(g.gl, ter, omt, H, Ht,
+                    mode == M_RK ? HOM::WANT_HT : mode == M_NEWTON && !need64 ? HOM::WANT_H : 0);
+      if (mode == M_COND) {
+        // the whole inverse in one elimination, and the largest column sum of
+        // its moduli: every column as one solve with that unit vector gives it
+        float an = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < N; ++j)
+          an = fmaxf(an, gsum<L, float>(g, act ? cabs2(cvt<float>(A[j * HOM::ROWL + grow])) : 0.f));
+        cond_anorm = an;
+        if (g.gl < HOM::ROWL)
+#pragma unroll 1
+          for (int j = 0; j < N; ++j)
+            A[(N + j) * HOM::ROWL + grow] = mk<df>(grow == j ? df(1) : df(0), df(0));
+        __syncwarp(g.meet);
+        sok = hom.template solve<MEET>(g, A, pv, 2 * N, dinv, col);
+#pragma unroll 1
+        for (int j = 0; j < N; ++j) {
+          const cx<df> x = A[(N + j) * HOM::ROWL + grow] * dinv;
+          if (col >= 0) sb[col] = x;
+          __syncwarp(g.meet);
+          cond_inorm = fmaxf(
+              cond_inorm,
+              gsum<L, float>(g, (act && col >= 0) ? cabs2(cvt<float>(sb[g.gl])) : 0.f));
+          __syncwarp(g.meet);
+        }
+        sol[0] = czero<df>();
+        stage = N - 1;
+      } else {
+        cx<df> rhs;
+        if (mode == M_RK)
+          rhs = -Ht;
+        else if (need64)
+          rhs = residual_rhs();
+        else
+          rhs = -H;
+        if (g.gl < HOM::ROWL) A[N * HOM::ROWL + grow] = rhs;
+        __syncwarp(g.meet);
+        sok = hom.template solve<MEET>(g, A, pv, N + 1, dinv, col);
+        sol[0] = A[N * HOM::ROWL + grow] * dinv;
+      }
+    } else {
+      cx<R> row[N + 1], x[N];  // (the evaluators read the point from shared memory)
       cx<R> H, Ht;
       hom.template eval<R>(x, g.gl, ter, omt, row, H, Ht);
       if (mode == M_RK) {
@@ -849,32 +905,17 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         const int grow = g.gl & (HOM::ROWL - 1);
         row[N] = mk<R>((grow < N && grow == stage) ? R(1) : R(0), R(0));
       } else if (!LOW && need64) {
-        if constexpr (COOP) {
-          const float4 v = reinterpret_cast<const float4*>(sm.sb)[g.gl];
-          row[N] = mk<R>(-v.x, -v.y);
-        } else if (MIXED && (mode == M_REFINE || !res64)) {
-          cx<float> Hf;
-          float sc;
-          hom.template residual_df<false, EP>(reinterpret_cast<const cdf*>(sm.vd), g.gl, te, Hf,
-                                              sc);
-          row[N] = cvt<R>(-Hf);
-        } else {
-          cx<double> H64;
-          double sc;
-          hom.template residual64<false, EP>(sm.vd, g.gl, te, 1.0 - te, H64, sc);
-          row[N] = cvt<R>(-H64);
-        }
+        row[N] = residual_rhs();
       } else {
         row[N] = -H;
       }
+      if constexpr (HOM::PARTS > 1)
+        sok = gj_solve_parts<N, R, HOM::ROWL, HOM::PARTS>(g, row, sol, col,
+                                                         reinterpret_cast<cx<R>*>(sm.pv),
+                                                         reinterpret_cast<cx<R>*>(sm.sb));
+      else
+        sok = gj_solve<N, 1, R, L, MEET>(g, row, sol, col, reinterpret_cast<cx<R>*>(sm.pv));
     }
-    bool sok;
-    if constexpr (HOM::PARTS > 1)
-      sok = gj_solve_parts<N, R, HOM::ROWL, HOM::PARTS>(g, row, sol, col,
-                                                       reinterpret_cast<cx<R>*>(sm.pv),
-                                                       reinterpret_cast<cx<R>*>(sm.sb));
-    else
-      sok = gj_solve<N, 1, R, L, MEET>(g, row, sol, col, reinterpret_cast<cx<R>*>(sm.pv));
     if (col >= 0) sb[col] = sol[0];
     __syncwarp(g.meet);
     const cx<R> d = act ? sb[g.gl] : czero<R>();
