@@ -72,8 +72,23 @@ struct Slot {
   hc_problem* problem = nullptr;
   std::vector<Request*> reqs;
   size_t bytes = 0;
+  Clock::time_point t_start;
   Pinned in, x, st, steps;
 };
+
+// A problem's batches so far: how many are in flight, when the last one started
+// and how long the last finished one took.
+struct Flow {
+  int inflight = 0;
+  Clock::time_point started;
+  Clock::duration took{0};
+};
+// Requests of a problem that is in flight wait for company up to an eighth of that
+// problem's last service time after its last start, and no longer than this: a
+// batch of several costs little more than one of one instance (the slowest path
+// sets the time), and an eighth is what a request can lose by it.  A problem that
+// is not in flight starts at once.
+constexpr auto kMostGather = std::chrono::milliseconds(4);
 
 }  // namespace
 
@@ -85,6 +100,7 @@ struct hc_server {
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
   std::map<hc_problem*, std::deque<Request*>> pending;
+  std::map<hc_problem*, Flow> flow;
   std::unordered_map<uint64_t, Request*> all;
   size_t bytes_inflight = 0;
   uint64_t next_id = 1;
@@ -120,6 +136,9 @@ void harvest(hc_server* s) {
     }
     hc_destroy(sl.batch);
     sl.batch = nullptr;
+    Flow& f = s->flow[sl.problem];
+    f.inflight -= 1;
+    f.took = now - sl.t_start;
     sl.reqs.clear();
     s->bytes_inflight -= sl.bytes;
     sl.bytes = 0;
@@ -150,6 +169,10 @@ void dispatch(hc_server* s) {
     Clock::time_point oldest;
     for (auto& kv : s->pending) {
       if (kv.second.empty()) continue;
+      const Flow& f = s->flow[kv.first];
+      if (f.inflight > 0 && (int)kv.second.size() < s->cfg.max_batch_instances &&
+          Clock::now() - f.started < std::min<Clock::duration>(f.took / 8, kMostGather))
+        continue;  // (in flight: the worker looks again within 50 us)
       if (waiting_problems > 1) {
         int held = 0;
         for (auto& sp : s->slots) held += (sp->busy && sp->problem == kv.first) ? 1 : 0;
@@ -217,6 +240,9 @@ void dispatch(hc_server* s) {
       r->state = 1;
       r->batch_instances = (int)k;
     }
+    Flow& f = s->flow[best];
+    f.inflight += 1;
+    f.started = sl.t_start = now;
     sl.busy = true;
     sl.batch = bt;
     sl.problem = best;
