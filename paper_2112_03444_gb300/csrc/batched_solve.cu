@@ -7,10 +7,15 @@
 // system, row i of [A | b] in lane i, Gauss-Jordan with partial pivoting, so
 // the back substitution is folded into the elimination.
 //
+// The groups of a warp run the elimination in step (make_group): with group masks
+// each ran it on its own (batch 100,000, FP32, together with the staging below:
+// n = 4 12.6 -> 8.5 us, n = 8 31 -> 28, n = 20 327 -> 281; batch 1000, n = 8 6.0 -> 4.6).
+//
 // Data path: a block's systems are contiguous in A (row-major, system after
 // system), so the block stages them through shared memory with consecutive
 // threads reading consecutive complex numbers (coalesced), then each lane
 // takes its row from shared memory; solutions go out the same way.
+#include <atomic>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -25,86 +30,140 @@ using hc::cx;
 
 constexpr int kThreads = 128;
 
-template <int N>
+// Lanes per system with one row per lane; D divides them (rows per lane: D, or
+// fewer where N leaves the last ones empty).
+//
+// FP64 is bound by its pipe (91 % busy at n = 13, batch 40,000, one row per lane),
+// and 38 % of its instructions are the reciprocals of the pivots, which cost a
+// warp the same whether its lanes belong to two systems or to eight.  With several
+// rows per lane a warp's reciprocals serve D times the systems: batch 100,000, us,
+// one row -> D rows: n = 5 289 -> 141, n = 8 494 -> 361, n = 12 1763 -> 977 (D = 4),
+// n = 13 1981 -> 1594, n = 20 7550 -> 6475 (D = 2; four rows of 13 or more entries
+// leave the registers).  A batch that does not fill the chip is bound by latency,
+// which the rows per lane lengthen (n = 13, batch 1000: 33 -> 46), so they are used
+// from 16 one-row warps per SM on: the two cross between 8 (n = 13, 20) and 14 (n = 4,
+// 8).  FP32 is bound by issue slots and its row updates: one row per lane (n = 20,
+// batch 100,000: 281 against 343 with two rows and two-wide updates).
+template <int N, class R>
+constexpr int wide_rows() {
+  return sizeof(R) == 4 || N > 24 ? 1 : N > 12 || N <= 2 ? 2 : 4;
+}
+constexpr int kFillWarps = 16;  // one-row warps per SM from which on
+template <int N, int D>
 constexpr int solve_lanes() {
-  return N <= 4 ? 4 : N <= 8 ? 8 : N <= 16 ? 16 : 32;
+  return (N <= 4 ? 4 : N <= 8 ? 8 : N <= 16 ? 16 : 32) / D;
 }
 
 // Shared memory of one block: the staged augmented matrices [G][N][N + 1],
 // then per group the two pivot-row buffers and the solution scatter buffer.
-template <int N, class R>
+template <int N, class R, int D>
 constexpr size_t solve_smem_bytes() {
-  constexpr int L = solve_lanes<N>(), G = kThreads / L;
+  constexpr int L = solve_lanes<N, D>(), G = kThreads / L;
   constexpr int S = (N + 2) & ~1;  // entries per pivot buffer (gj_solve, NR = 1)
-  return sizeof(cx<R>) * ((size_t)G * N * (N + 1) + (size_t)G * 2 * S + (size_t)G * L);
+  return sizeof(cx<R>) * ((((size_t)G * N * (N + 1) + 1) & ~(size_t)1) + (size_t)G * 2 * S +
+                          (size_t)G * N);
 }
 
-template <int N, class R>
+template <int N, class R, int D>
 __global__ void __launch_bounds__(kThreads) batched_solve_kernel(int64_t batch,
                                                                  const cx<R>* __restrict__ A,
                                                                  const cx<R>* __restrict__ b,
                                                                  cx<R>* __restrict__ x,
                                                                  int32_t* __restrict__ info) {
-  constexpr int L = solve_lanes<N>(), G = kThreads / L, W = N + 1;
+  constexpr int L = solve_lanes<N, D>(), G = kThreads / L, W = N + 1;
+  constexpr int ROWS = (N + L - 1) / L;
   constexpr int S = (N + 2) & ~1;
   extern __shared__ __align__(16) unsigned char smem[];
   cx<R>* stage = reinterpret_cast<cx<R>*>(smem);
-  cx<R>* pvbuf = stage + (size_t)G * N * W;
+  cx<R>* pvbuf = stage + (((size_t)G * N * W + 1) & ~(size_t)1);
   cx<R>* sbuf = pvbuf + (size_t)G * 2 * S;
-  const hc::Group g = hc::make_group<L>();
+  const hc::Group g = hc::make_group<L, true>();
   const int grp = threadIdx.x / L;
   cx<R>* pv = pvbuf + grp * 2 * S;
-  cx<R>* sb = sbuf + grp * L;
+  cx<R>* sb = sbuf + grp * N;
   for (int64_t base = (int64_t)blockIdx.x * G; base < batch; base += (int64_t)gridDim.x * G) {
     const int cnt = (int)((batch - base) < G ? (batch - base) : G);
-    // coalesced staging of the block's matrices and right-hand sides
+    // Coalesced staging of the block's matrices and right-hand sides: row r of the
+    // block (N entries) lands at r W, so entry idx at idx + idx / N.
     const cx<R>* Ab = A + base * N * N;
-    for (int idx = threadIdx.x; idx < cnt * N * N; idx += kThreads) {
-      const int sys = idx / (N * N), r = idx % (N * N);
-      stage[(sys * N + r / N) * W + r % N] = Ab[idx];
-    }
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < cnt * N * N; idx += kThreads)
+      stage[idx + (unsigned)idx / N] = Ab[idx];
     const cx<R>* bb = b + base * N;
-    for (int idx = threadIdx.x; idx < cnt * N; idx += kThreads)
-      stage[(idx / N * N + idx % N) * W + N] = bb[idx];
+    for (int idx = threadIdx.x; idx < cnt * N; idx += kThreads) stage[idx * W + N] = bb[idx];
     __syncthreads();
-    cx<R> a[W];
+    cx<R> a[ROWS][W];
     const bool live = grp < cnt;
 #pragma unroll
-    for (int j = 0; j < W; ++j)
-      a[j] = (live && g.gl < N) ? stage[(grp * N + g.gl) * W + j] : hc::czero<R>();
+    for (int q = 0; q < ROWS; ++q)
+#pragma unroll
+      for (int j = 0; j < W; ++j)
+        a[q][j] = (live && g.gl + q * L < N) ? stage[(grp * N + g.gl + q * L) * W + j]
+                                             : hc::czero<R>();
     __syncthreads();  // the stage is free for the next round once every row is in registers
+    cx<R> sol[ROWS];
+    int col[ROWS];
+    bool ok;
+    if constexpr (ROWS == 1)
+      ok = hc::gj_solve<N, 1, R, L, true>(g, a[0], sol, col[0], pv);
+    else
+      ok = hc::gj_solve_rows<N, L, ROWS, R>(g, a, sol, col, pv);
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+      if (col[q] >= 0) sb[col[q]] = sol[q];
+    __syncwarp();
     if (live) {
-      cx<R> sol[1];
-      int col;
-      const bool ok = hc::gj_solve<N, 1, R>(g, a, sol, col, pv);
-      if (col >= 0) sb[col] = sol[0];
-      __syncwarp(g.mask);
-      if (g.gl < N) x[(base + grp) * N + g.gl] = sb[g.gl];
+#pragma unroll
+      for (int q = 0; q < ROWS; ++q)
+        if (g.gl + q * L < N) x[(base + grp) * N + g.gl + q * L] = sb[g.gl + q * L];
       if (g.gl == 0 && info) info[base + grp] = ok ? 0 : 1;
-      __syncwarp(g.mask);
     }
+    __syncwarp();
   }
 }
+
+constexpr int kMaxDevices = 64;
 
 struct SolveRef {
   const void* fn;
   size_t smem;
-  int per_block;
+  int per_block, per_sm;  // systems per block, resident blocks per SM (0: refused)
 };
 
-template <int N, class R>
-SolveRef solve_ref() {
-  return SolveRef{reinterpret_cast<const void*>(&batched_solve_kernel<N, R>),
-                  solve_smem_bytes<N, R>(), kThreads / solve_lanes<N>()};
+// The occupancy query costs as much as the launch of a small batch: once per
+// kernel and device.
+template <int N, class R, int D>
+SolveRef solve_ref(int dev) {
+  static std::atomic<int> known[kMaxDevices];
+  SolveRef k{reinterpret_cast<const void*>(&batched_solve_kernel<N, R, D>),
+             solve_smem_bytes<N, R, D>(), kThreads / solve_lanes<N, D>(),
+             dev < kMaxDevices ? known[dev].load(std::memory_order_acquire) : 0};
+  if (k.per_sm > 0) return k;
+  if (k.smem > 48 * 1024 &&
+      cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) !=
+          cudaSuccess)
+    return k;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k.per_sm, k.fn, kThreads, k.smem) !=
+      cudaSuccess)
+    k.per_sm = 0;
+  else if (k.per_sm < 1)
+    k.per_sm = 1;
+  if (dev < kMaxDevices) known[dev].store(k.per_sm, std::memory_order_release);
+  return k;
 }
 
 template <class R, int N = 1>
-SolveRef solve_dispatch(int n) {
+SolveRef solve_dispatch(int n, int64_t batch, int sms, int dev) {
   if constexpr (N > 32) {
-    return SolveRef{nullptr, 0, 0};
+    return SolveRef{nullptr, 0, 0, 0};
   } else {
-    if (n == N) return solve_ref<N, R>();
-    return solve_dispatch<R, N + 1>(n);
+    if (n == N) {
+      constexpr int D = wide_rows<N, R>();
+      if (D > 1 && batch >= (int64_t)kFillWarps * sms * (32 / solve_lanes<N, 1>()))
+        return solve_ref<N, R, D>(dev);
+      return solve_ref<N, R, 1>(dev);
+    }
+    return solve_dispatch<R, N + 1>(n, batch, sms, dev);
   }
 }
 
@@ -117,29 +176,26 @@ extern "C" hc_status hc_batched_solve(int32_t n, int64_t batch, int32_t fp32, co
     return HC_ERR_INVALID;
   }
   if (batch == 0) return HC_OK;
-  const SolveRef k = fp32 ? solve_dispatch<float>(n) : solve_dispatch<double>(n);
+  cudaGetLastError();
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    hc::set_last_error("hc_batched_solve: device query failed");
+    return HC_ERR_CUDA;
+  }
+  const SolveRef k =
+      fp32 ? solve_dispatch<float>(n, batch, sms, dev) : solve_dispatch<double>(n, batch, sms, dev);
   if (!k.fn) {
     hc::set_last_error("hc_batched_solve: no kernel for this size");
     return HC_ERR_UNSUPPORTED;
   }
-  cudaGetLastError();
-  if (k.smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) !=
-          cudaSuccess) {
-    hc::set_last_error("hc_batched_solve: shared-memory attribute refused");
-    return HC_ERR_CUDA;
-  }
-  int dev = 0, sms = 0, per_sm = 1;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, kThreads, k.smem) !=
-          cudaSuccess) {
-    hc::set_last_error("hc_batched_solve: device query failed");
+  if (k.per_sm < 1) {
+    hc::set_last_error("hc_batched_solve: shared-memory attribute or occupancy query refused");
     return HC_ERR_CUDA;
   }
   // one wave of resident blocks at most; each block strides over the batch
   const int64_t want = (batch + k.per_block - 1) / k.per_block;
-  const int64_t cap = (int64_t)(per_sm < 1 ? 1 : per_sm) * sms;
+  const int64_t cap = (int64_t)k.per_sm * sms;
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   void* args[] = {&batch, &A, &b, &x, &info};
   if (cudaLaunchKernel(k.fn, dim3(grid), dim3(kThreads), args, k.smem,

@@ -254,6 +254,100 @@ __device__ __forceinline__ bool gj_solve(const Group& g, cx<R> (&a)[N + NR], cx<
   return (lo & ~31u) != 0u && (hi & ~31u) < 0x7f800000u;
 }
 
+// The same elimination with ROWS rows per lane (lane gl of L: rows gl, gl + L, ..),
+// for the batched solve: a warp then holds ROWS times the systems, and the pivot
+// search, the reciprocal and the pivot row's broadcast of a step are shared by all
+// of them.  In a lane the largest candidate is found first and only its reciprocal
+// is formed.  The same operations per entry, hence the same results.  All lanes of
+// the warp take part.
+template <int N, int L, int ROWS, class R>
+__device__ __forceinline__ bool gj_solve_rows(const Group& g, cx<R> (&a)[ROWS][N + 1],
+                                              cx<R> (&sol)[ROWS], int (&col)[ROWS], cx<R>* pv) {
+  constexpr int W = N + 1;
+  constexpr int S = (W + 1) & ~1;
+  bool used[ROWS];
+  cx<R> dinv[ROWS];
+#pragma unroll
+  for (int q = 0; q < ROWS; ++q) {
+    used[q] = g.gl + q * L >= N;
+    dinv[q] = mk<R>(R(1), R(0));
+    col[q] = -1;
+  }
+  unsigned lo = 0xffffffffu, hi = 0u;
+  auto search = [&](int k, cx<R>& inv, unsigned& kmax) {
+    cx<R> z = a[0][k];
+    unsigned key = 0u;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      const unsigned kq = used[q] ? 0u
+                                  : ((__float_as_uint((float)cabs1(a[q][k])) & ~31u) |
+                                     (unsigned)(31 - (g.gl + q * L)));
+      if (q > 0 && kq > key) z = a[q][k];
+      key = max(key, kq);
+    }
+    inv = crecip(z);
+    kmax = gmaxu<L, true>(g, key);
+  };
+  cx<R> inv;
+  unsigned kmax;
+  search(0, inv, kmax);
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    lo = min(lo, kmax);
+    hi = max(hi, kmax);
+    const int prow = 31 - (int)(kmax & 31u);
+    cx<R>* buf = pv + (k & 1) * S;
+    const int j0 = k & ~1;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      if (prow == g.gl + q * L) {
+        if constexpr (sizeof(R) == 4) {
+#pragma unroll
+          for (int j = j0; j < W; j += 2) {
+            const cx<R> v0 = (j == k) ? inv : a[q][j];
+            const cx<R> v1 =
+                (j + 1 == k) ? inv : (j + 1 < W ? a[q][j + 1 < W ? j + 1 : 0] : czero<R>());
+            reinterpret_cast<float4*>(buf)[j >> 1] = make_float4(v0.re, v0.im, v1.re, v1.im);
+          }
+        } else {
+#pragma unroll
+          for (int j = k; j < W; ++j) buf[j] = (j == k) ? inv : a[q][j];
+        }
+        used[q] = true;
+        dinv[q] = inv;
+        col[q] = k;
+      }
+    }
+    __syncwarp();
+    cx<R> row_p[W];
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+      for (int j = j0; j < W; j += 2) {
+        const float4 v = reinterpret_cast<const float4*>(buf)[j >> 1];
+        row_p[j] = mk<R>(v.x, v.y);
+        if (j + 1 < W) row_p[j + 1 < W ? j + 1 : 0] = mk<R>(v.z, v.w);
+      }
+    } else {
+#pragma unroll
+      for (int j = k; j < W; ++j) row_p[j] = buf[j];
+    }
+    cx<R> l[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      l[q] = prow == g.gl + q * L ? czero<R>() : a[q][k] * row_p[k];
+      a[q][k + 1] = cfms(l[q], row_p[k + 1], a[q][k + 1]);
+    }
+    if (k + 1 < N) search(k + 1 < N ? k + 1 : 0, inv, kmax);
+#pragma unroll
+    for (int j = k + 2; j < W; ++j)
+#pragma unroll
+      for (int q = 0; q < ROWS; ++q) a[q][j] = cfms(l[q], row_p[j], a[q][j]);
+  }
+#pragma unroll
+  for (int q = 0; q < ROWS; ++q) sol[q] = a[q][N] * dinv[q];
+  return (lo & ~31u) != 0u && (hi & ~31u) < 0x7f800000u;
+}
+
 // The same elimination for groups whose rows are replicated over PARTS
 // lanes (one path per warp with the evaluation split over the warp, L0 =
 // lanes per replica): lane gl holds row r = gl mod L0 and owns the columns j
