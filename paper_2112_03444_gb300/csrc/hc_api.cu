@@ -372,8 +372,10 @@ int graded_index(int n, const std::vector<int>& vars /* sorted ascending */) {
   return idx;
 }
 
-struct DeviceBuf {
+// A pinned host buffer of the pool (HostPool)
+struct HostBuf {
   void* p = nullptr;
+  size_t cap = 0;
 };
 
 }  // namespace
@@ -427,6 +429,7 @@ struct hc_problem {
   uint8_t* d_sign = nullptr;
   double2* d_p0 = nullptr;
   double2* d_start = nullptr;
+  bool counted = false;  // among the problems that keep the memory pools filled
 };
 
 struct hc_batch {
@@ -447,7 +450,7 @@ struct hc_batch {
     size_t bytes;
   };
   std::vector<HostCopy> copies;
-  std::vector<void*> pinned;
+  std::vector<HostBuf> pinned;
   bool owns_ctl = false;            // h_ctl from the pinned pool (else a plan's)
   bool owns_kernel_events = false;  // evk* created for this batch (else a plan's)
   int64_t step_budget = 0;
@@ -487,6 +490,115 @@ void pinned_slot_put(void* q) {
   PinnedPool& pp = pinned_pool();
   std::lock_guard<std::mutex> lk(pp.mu);
   pp.free_slots.push_back(q);
+}
+
+// Pinned staging buffers of the batches' host outputs, kept between batches:
+// allocating and freeing pinned memory took longer than a small batch's tracking
+// (one quadratic n = 6 system, numpy in and out: 1069 -> 875 us, with the device
+// pool and the wait below).  Buffers are powers
+// of two from 4 KiB to 16 MiB (larger ones are not kept), at most 128 MiB lie
+// idle, and all idle ones are given back with the last problem.
+struct HostPool {
+  static constexpr size_t kSmallest = 4096, kLargest = size_t(16) << 20;
+  static constexpr size_t kMostIdle = size_t(128) << 20;
+  std::mutex mu;
+  std::map<size_t, std::vector<void*>> idle;
+  size_t idle_bytes = 0;
+};
+HostPool& host_pool() {
+  static HostPool pool;
+  return pool;
+}
+HostBuf host_buf_get(size_t bytes) {
+  HostBuf b;
+  b.cap = bytes;
+  if (bytes <= HostPool::kLargest) {
+    b.cap = HostPool::kSmallest;
+    while (b.cap < bytes) b.cap *= 2;
+    HostPool& pool = host_pool();
+    std::lock_guard<std::mutex> lk(pool.mu);
+    auto it = pool.idle.find(b.cap);
+    if (it != pool.idle.end() && !it->second.empty()) {
+      b.p = it->second.back();
+      it->second.pop_back();
+      pool.idle_bytes -= b.cap;
+      return b;
+    }
+  }
+  if (cudaHostAlloc(&b.p, b.cap, cudaHostAllocPortable) != cudaSuccess) b.p = nullptr;
+  return b;
+}
+// (no work that uses the buffer may be in flight)
+void host_buf_put(const HostBuf& b) {
+  if (!b.p) return;
+  if (b.cap <= HostPool::kLargest) {
+    HostPool& pool = host_pool();
+    std::lock_guard<std::mutex> lk(pool.mu);
+    if (pool.idle_bytes + b.cap <= HostPool::kMostIdle) {
+      pool.idle[b.cap].push_back(b.p);
+      pool.idle_bytes += b.cap;
+      return;
+    }
+  }
+  cudaFreeHost(b.p);
+}
+
+// Device memory of the batches: a pool of its own per device, which keeps up to
+// 256 MiB between batches (the default pool returns everything at the next
+// synchronisation, and mapping it again costs a small batch more than its kernels)
+// and gives it back with the last problem.
+struct DevicePools {
+  static constexpr int kDevices = 64;
+  std::mutex mu;
+  cudaMemPool_t pool[kDevices] = {};
+  bool tried[kDevices] = {};
+  int problems = 0;
+};
+DevicePools& device_pools() {
+  static DevicePools d;
+  return d;
+}
+cudaError_t pool_malloc(void** q, size_t bytes, int dev, cudaStream_t st) {
+  cudaMemPool_t pool = nullptr;
+  if (dev >= 0 && dev < DevicePools::kDevices) {
+    DevicePools& d = device_pools();
+    std::lock_guard<std::mutex> lk(d.mu);
+    if (!d.tried[dev]) {
+      d.tried[dev] = true;
+      cudaMemPoolProps props;
+      std::memset(&props, 0, sizeof(props));
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      uint64_t keep = uint64_t(256) << 20;
+      if (cudaMemPoolCreate(&d.pool[dev], &props) != cudaSuccess) {
+        d.pool[dev] = nullptr;
+        cudaGetLastError();
+      } else {
+        cudaMemPoolSetAttribute(d.pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+      }
+    }
+    pool = d.pool[dev];
+  }
+  if (!pool) return cudaMallocAsync(q, bytes, st);
+  return cudaMallocFromPoolAsync(q, bytes, pool, st);
+}
+// A problem comes (+1) or goes (-1); with the last one the pools are emptied.
+void count_problem(int by) {
+  DevicePools& d = device_pools();
+  {
+    std::lock_guard<std::mutex> lk(d.mu);
+    d.problems += by;
+    if (d.problems > 0) return;
+    for (cudaMemPool_t pool : d.pool)
+      if (pool) cudaMemPoolTrimTo(pool, 0);
+  }
+  HostPool& h = host_pool();
+  std::lock_guard<std::mutex> lk(h.mu);
+  for (auto& kv : h.idle)
+    for (void* q : kv.second) cudaFreeHost(q);
+  h.idle.clear();
+  h.idle_bytes = 0;
 }
 
 // High-priority streams for the re-tracking branch of hc_track_batch, handed
@@ -935,6 +1047,7 @@ void free_problem(hc_problem* p) {
   cudaFree(p->d_p0);
   cudaFree(p->d_start);
   p->magic = 0;
+  if (p->counted) count_problem(-1);
   delete p;
 }
 
@@ -1286,6 +1399,8 @@ hc_status hc_create_problem(const hc_problem_desc* d, hc_problem** out) {
       free_problem(p);
       return st;
     }
+    count_problem(1);
+    p->counted = true;
     *out = p;
     return HC_OK;
   }
@@ -1305,6 +1420,8 @@ hc_status hc_create_problem(const hc_problem_desc* d, hc_problem** out) {
     free_problem(p);
     return st;
   }
+  count_problem(1);
+  p->counted = true;
   *out = p;
   return HC_OK;
 }
@@ -1712,7 +1829,7 @@ void release_batch(hc_batch* bt) {
   admit_release(bt->p ? bt->p->device : 0, bt->admission);
   bt->admission.reset();
   for (void* q : bt->dev) cudaFree(q);
-  for (void* q : bt->pinned) cudaFreeHost(q);
+  for (const HostBuf& q : bt->pinned) host_buf_put(q);
   if (bt->h_ctl && bt->owns_ctl) pinned_slot_put(bt->h_ctl);
   for (cudaEvent_t e : {bt->ev0, bt->ev1})
     if (e) cudaEventDestroy(e);
@@ -1739,13 +1856,13 @@ hc_status setup_outputs(hc_batch* bt, const hc_batch_desc* b, int n, int64_t ite
       if (is_pinned_host(user)) {
         bt->copies.push_back({user, nullptr, bytes});
       } else {
-        void* pin;
-        if (cudaMallocHost(&pin, bytes) != cudaSuccess) {
-          set_err("cudaMallocHost failed");
+        const HostBuf pin = host_buf_get(bytes);
+        if (!pin.p) {
+          set_err("cudaHostAlloc failed");
           return HC_ERR_OOM;
         }
         bt->pinned.push_back(pin);
-        bt->copies.push_back({user, pin, bytes});
+        bt->copies.push_back({user, pin.p, bytes});
       }
       d2h.push_back(*dptr);
     }
@@ -1835,7 +1952,7 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
     return s;
   };
   std::function<hc_status(size_t, void**)> dalloc = [&](size_t bytes, void** q) -> hc_status {
-    cudaError_t e = cudaMallocAsync(q, std::max<size_t>(bytes, 16), st);
+    cudaError_t e = pool_malloc(q, std::max<size_t>(bytes, 16), p->device, st);
     if (e != cudaSuccess) {
       set_err(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
       return e == cudaErrorMemoryAllocation ? HC_ERR_OOM : HC_ERR_CUDA;
@@ -1870,14 +1987,14 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
     HC_TRY(dalloc(bytes, &q));
     // the caller may free path_ids on return: copy through a pinned buffer
     // the batch owns, so the upload stays asynchronous
-    void* pin = nullptr;
-    if (cudaMallocHost(&pin, bytes) != cudaSuccess) {
-      set_err("cudaMallocHost failed");
+    const HostBuf pin = host_buf_get(bytes);
+    if (!pin.p) {
+      set_err("cudaHostAlloc failed");
       return fail(HC_ERR_OOM);
     }
     bt->pinned.push_back(pin);
-    std::memcpy(pin, b->path_ids, bytes);
-    HC_TRYCUDA(cudaMemcpyAsync(q, pin, bytes, cudaMemcpyHostToDevice, st));
+    std::memcpy(pin.p, b->path_ids, bytes);
+    HC_TRYCUDA(cudaMemcpyAsync(q, pin.p, bytes, cudaMemcpyHostToDevice, st));
     B.path_ids = (const int64_t*)q;
   }
   // ---- inputs on the device
@@ -2153,14 +2270,14 @@ hc_status hc_plan_run(hc_plan* pl, const hc_batch_desc* b, hc_batch** out) {
     if (devptrs || is_pinned_host(o.user) || is_device_ptr(o.user)) {
       HC_TRYCUDA(cudaMemcpyAsync(o.user, o.dev, o.bytes, cudaMemcpyDefault, st));
     } else {
-      void* pin;
-      if (cudaMallocHost(&pin, o.bytes) != cudaSuccess) {
-        set_err("cudaMallocHost failed");
+      const HostBuf pin = host_buf_get(o.bytes);
+      if (!pin.p) {
+        set_err("cudaHostAlloc failed");
         return fail(HC_ERR_OOM);
       }
       bt->pinned.push_back(pin);
-      bt->copies.push_back({o.user, pin, o.bytes});
-      HC_TRYCUDA(cudaMemcpyAsync(pin, o.dev, o.bytes, cudaMemcpyDeviceToHost, st));
+      bt->copies.push_back({o.user, pin.p, o.bytes});
+      HC_TRYCUDA(cudaMemcpyAsync(pin.p, o.dev, o.bytes, cudaMemcpyDeviceToHost, st));
     }
   }
   HC_TRYCUDA(cudaEventRecord(bt->ev1, st));
@@ -2191,7 +2308,12 @@ hc_status hc_poll(hc_batch* b, int64_t timeout_us, hc_batch_result* r) {
                           std::chrono::steady_clock::now() - t0)
                           .count();
       if (timeout_us > 0 && el >= timeout_us) return HC_PENDING;
-      std::this_thread::sleep_for(std::chrono::microseconds(el < 200 ? 2 : 50));
+      // a sleep of any length takes 50 us and more (timer slack), a tenth of a small
+      // batch: yield for the first 2 ms
+      if (el < 2000)
+        std::this_thread::yield();
+      else
+        std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
     for (auto& c : b->copies)
       if (c.pinned) std::memcpy(c.dst, c.pinned, c.bytes);
