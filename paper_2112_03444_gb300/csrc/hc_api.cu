@@ -208,8 +208,8 @@ __global__ void dedupe_list_kernel(int64_t paths, int n, const float2* __restric
                                    const uint8_t* __restrict__ status, float tol,
                                    const int64_t* __restrict__ list,
                                    const unsigned long long* list_count, int64_t* out_list,
-                                   unsigned long long* out_count, double* t_io, int n_group,
-                                   const uint32_t* __restrict__ group) {
+                                   int out_step, unsigned long long* out_count, double* t_io,
+                                   int n_group, const uint32_t* __restrict__ group) {
   const int lane = threadIdx.x & 31;
   const int64_t total = (int64_t)*list_count;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
@@ -239,7 +239,7 @@ __global__ void dedupe_list_kernel(int64_t paths, int n, const float2* __restric
       t_io[a] = 0.0;
       if ((status[a] & 0x7f) != HC_PATH_SINGULAR) {
         const unsigned long long pos = atomicAdd(out_count, 1ull);
-        out_list[pos] = a;
+        out_list[(int64_t)pos * out_step] = a;
       }
     }
   }
@@ -438,6 +438,7 @@ struct hc_batch {
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   cudaEvent_t evk0 = nullptr, evk1 = nullptr, evk2 = nullptr;  // around the tracking launches
+  cudaEvent_t evf = nullptr, evj = nullptr;  // fork and join of the early re-tracking
   int64_t n_inst = 0, items = 0;
   bool done = false;
   std::vector<void*> dev;  // device allocations (stream-ordered)
@@ -472,6 +473,7 @@ PinnedPool& pinned_pool() {
 // control words of a batch: [0] queue [1] FP64 queue [2] FP64 list count
 // [3..5] FP64 steps [6] re-track queue [7] re-track list count [8..15]
 // summary [16] untracked paths [17] steps counted against the budget
+// [20] [21] late FP64 list count and queue
 constexpr int kCtlWords = 24;
 constexpr size_t kCtlBytes = sizeof(unsigned long long) * kCtlWords;
 void* pinned_slot_get() {
@@ -610,7 +612,7 @@ void count_problem(int by) {
 // skipped (nullptr only if every creation failed: the caller then runs the
 // re-tracking on its own stream).
 cudaStream_t retrack_stream(int device) {
-  constexpr int kPerDevice = 16, kMaxDev = 64;
+  constexpr int kPerDevice = 32, kMaxDev = 64;
   static std::mutex mu;
   static cudaStream_t streams[kMaxDev][kPerDevice] = {};
   static bool tried[kMaxDev] = {};
@@ -1555,8 +1557,9 @@ int main_threads(const hc_settings& s) { return s.block_threads ? s.block_thread
 // tracking launch and the summary after the re-tracking.  Under stream
 // capture the timing events become event-record nodes of the graph
 // (external), the fork/join events only graph edges.
+// fork2 and join2 order the early re-tracking (stream hs2).
 struct EnqEvents {
-  cudaEvent_t ek0, ek1, ek2, fork, join;
+  cudaEvent_t ek0, ek1, ek2, fork, join, fork2, join2;
   bool capture;
 };
 
@@ -1565,7 +1568,7 @@ struct EnqEvents {
 // copy of the control words to B.h_ctl.  Allocates nothing and never waits
 // on the host, so it can be captured into a CUDA graph.
 hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStream_t st,
-                          cudaStream_t hs, const EnqEvents& ev) {
+                          cudaStream_t hs, cudaStream_t hs2, const EnqEvents& ev) {
   auto mark = [&](cudaEvent_t e, cudaStream_t s) {
     return ev.capture ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal)
                       : cudaEventRecord(e, s);
@@ -1623,6 +1626,10 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   cm.be_out = tbe;
   cm.esc_list = B.esc_list;
   cm.esc_count = B.d_ctl + 2;
+  int64_t* late = B.esc_list ? B.esc_list + (items - 1) : nullptr;
+  cm.items_step = 1;
+  cm.late_end = late;
+  cm.late_count = B.d_ctl + 20;
   cm.t_io = B.t_io;
   cm.x32_out = B.x32;
   cm.dup_list = B.dup_list;
@@ -1635,7 +1642,13 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   // and FP64 tolerances.  Whatever still fails or collides after that tier,
   // step-size failures and suspect-condition endpoints (esc_list, ctl[2])
   // run in the all-FP64 kernel: from t = 0, from the last accepted point, or
-  // only the refinement and condition at t = 1.
+  // only the refinement and condition at t = 1.  The step-size failures of the
+  // tracking launch (ctl[2] of them, often the longest paths of the batch) depend
+  // on neither the duplicate check nor the tier before and are re-tracked beside
+  // them on hs2; the others (from the end of esc_list, ctl[20]) behind that
+  // tier.  Measured, re-tracking time in ms: trifocal (4 scenes, at most 800 steps)
+  // 327 -> 266, cubic n = 8 (16 systems) 17.5 -> 13.3, P3P (3000) 12.4 -> 9.6, quadratic
+  // n = 12 (16) 4.7 -> 3.1.
   hc::LaunchCommon cd = cm;
   cd.count_dev = B.d_ctl + 7;
   cd.items = B.dup_list;
@@ -1647,6 +1660,7 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   hc::LaunchCommon ce = cm;
   ce.count_dev = B.d_ctl + 2;
   ce.items = B.esc_list;
+  ce.late_end = nullptr;
   ce.queue = B.d_ctl + 1;
   ce.esc_list = nullptr;
   ce.x32_out = nullptr;
@@ -1654,10 +1668,30 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   ce.spread = 1;
   ce.dup_list = nullptr;
   ce.dup_count = nullptr;
+  if (!hs) hs = st;
+  if (!hs2) hs2 = hs;
+  hc::LaunchCommon cl = ce;
+  cl.count_dev = B.d_ctl + 20;
+  cl.items = late;
+  cl.items_step = -1;
+  cl.queue = B.d_ctl + 21;
+  // the early launch: behind the duplicate check, so that the tier after it, on
+  // hs, is launched at the same time and both share the SMs
+  auto fork_early = [&]() -> hc_status {
+    if (hs2 == hs) return HC_OK;
+    HC_CUDA(cudaEventRecord(ev.fork2, hs));
+    HC_CUDA(cudaStreamWaitEvent(hs2, ev.fork2, 0));
+    return HC_OK;
+  };
+  auto join_early = [&]() -> hc_status {
+    if (hs2 == hs) return HC_OK;
+    HC_CUDA(cudaEventRecord(ev.join2, hs2));
+    HC_CUDA(cudaStreamWaitEvent(hs, ev.join2, 0));
+    return HC_OK;
+  };
   // the count of re-tracked items is only known on the device: the grid
   // covers up to every item (capped at full occupancy by the launcher)
   const int64_t esc_groups = items;
-  if (!hs) hs = st;
   auto dedupe = [&]() -> hc_status {
     HC_CUDA(cudaStreamWaitEvent(hs, ev.capture ? ev.fork : ev.ek1, 0));
     HC_CUDA(dedupe_all(items, paths, n, B.x32, tst, 1e-6f, B.dup_list, B.d_ctl + 7, B.t_io,
@@ -1669,8 +1703,8 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   auto dedupe_again = [&]() -> hc_status {
     const int grid = (int)std::min<int64_t>((items + 7) / 8, 1024);  // 8 warps per block
     dedupe_list_kernel<<<std::max(grid, 1), 256, 0, hs>>>(paths, n, B.x32, tst, 1e-6f,
-                                                         B.dup_list, B.d_ctl + 7, B.esc_list,
-                                                         B.d_ctl + 2, B.t_io, n_group, group);
+                                                         B.dup_list, B.d_ctl + 7, late, -1,
+                                                         B.d_ctl + 20, B.t_io, n_group, group);
     HC_CUDA(cudaGetLastError());
     return HC_OK;
   };
@@ -1724,17 +1758,22 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
     if (escalate) {
       if (ev.capture) HC_CUDA(cudaEventRecord(ev.fork, st));
       if ((rc = dedupe()) != HC_OK) return rc;
+      if ((rc = fork_early()) != HC_OK) return rc;
       hc::TermArgs td = ta;
       td.c = cd;
       const int th = fit(k, hc::retrack_threads(k.lanes));
       if ((rc = launch_generic(k, &td, smem_of(k, th), esc_groups, hs, th)) != HC_OK) return rc;
-      if ((rc = dedupe_again()) != HC_OK) return rc;
       hc::TermArgs te = ta;
       te.c = ce;
       const hc::KernelRef k64 = hc::term_kernel(n, hc::last_tier_precision(p->s), 0);
       const int th64 = fit(k64, hc::retrack_threads(k64.lanes));
+      if ((rc = launch_generic(k64, &te, smem_of(k64, th64), esc_groups, hs2, th64)) != HC_OK)
+        return rc;
+      if ((rc = dedupe_again()) != HC_OK) return rc;
+      te.c = cl;
       if ((rc = launch_generic(k64, &te, smem_of(k64, th64), esc_groups, hs, th64)) != HC_OK)
         return rc;
+      if ((rc = join_early()) != HC_OK) return rc;
       HC_CUDA(mark(ev.ek2, hs));
       if (ev.capture) HC_CUDA(cudaEventRecord(ev.join, hs));
       HC_CUDA(cudaStreamWaitEvent(st, ev.capture ? ev.join : ev.ek2, 0));
@@ -1772,14 +1811,19 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
       hc::DenseArgs dd = a;
       dd.c = cd;
       const hc::KernelRef kr = retrack_kernel(p->deg, n, HC_PREC_MIXED);
+      if ((rc = fork_early()) != HC_OK) return rc;
       if ((rc = launch_tracker(kr, dd, esc_groups, hs, hc::retrack_threads(kr.lanes))) != HC_OK)
         return rc;
-      if ((rc = dedupe_again()) != HC_OK) return rc;
       hc::DenseArgs e = a;
       e.c = ce;
       const hc::KernelRef k64 = retrack_kernel(p->deg, n, hc::last_tier_precision(p->s));
+      if ((rc = launch_tracker(k64, e, esc_groups, hs2, hc::retrack_threads(k64.lanes))) != HC_OK)
+        return rc;
+      if ((rc = dedupe_again()) != HC_OK) return rc;
+      e.c = cl;
       if ((rc = launch_tracker(k64, e, esc_groups, hs, hc::retrack_threads(k64.lanes))) != HC_OK)
         return rc;
+      if ((rc = join_early()) != HC_OK) return rc;
       HC_CUDA(mark(ev.ek2, hs));
       if (ev.capture) HC_CUDA(cudaEventRecord(ev.join, hs));
       HC_CUDA(cudaStreamWaitEvent(st, ev.capture ? ev.join : ev.ek2, 0));
@@ -1834,7 +1878,7 @@ void release_batch(hc_batch* bt) {
   for (cudaEvent_t e : {bt->ev0, bt->ev1})
     if (e) cudaEventDestroy(e);
   if (bt->owns_kernel_events)
-    for (cudaEvent_t e : {bt->evk0, bt->evk1, bt->evk2})
+    for (cudaEvent_t e : {bt->evk0, bt->evk1, bt->evk2, bt->evf, bt->evj})
       if (e) cudaEventDestroy(e);
   bt->magic = 0;
   delete bt;
@@ -1946,7 +1990,7 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
   const int64_t items = bt->items;
   cudaStream_t st = bt->stream;
   auto fail = [&](hc_status s) {
-    cudaStreamSynchronize(st);
+    cudaDeviceSynchronize();  // the re-tracking streams may hold launches of the batch
     release_batch(bt);
     if (cur != p->device) cudaSetDevice(cur);
     return s;
@@ -1975,6 +2019,8 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
   } while (0)
   for (cudaEvent_t* e : {&bt->ev0, &bt->ev1, &bt->evk0, &bt->evk1, &bt->evk2})
     HC_TRYCUDA(cudaEventCreate(e));
+  for (cudaEvent_t* e : {&bt->evf, &bt->evj})
+    HC_TRYCUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   bt->owns_kernel_events = true;
   HC_TRYCUDA(cudaEventRecord(bt->ev0, st));
 
@@ -2038,8 +2084,9 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
   B.h_ctl = bt->h_ctl;
   bt->d_ctl = B.d_ctl;
   // ---- the computation
-  const EnqEvents ev{bt->evk0, bt->evk1, bt->evk2, nullptr, nullptr, false};
-  HC_TRY(enqueue_compute(p, bt->n_inst, B, st, retrack_stream(p->device), ev));
+  const EnqEvents ev{bt->evk0, bt->evk1, bt->evk2, nullptr, nullptr, bt->evf, bt->evj, false};
+  const cudaStream_t hs = retrack_stream(p->device);
+  HC_TRY(enqueue_compute(p, bt->n_inst, B, st, hs, retrack_stream(p->device), ev));
   for (size_t i = 0; i < bt->copies.size(); ++i) {
     void* dst = bt->copies[i].pinned ? bt->copies[i].pinned : bt->copies[i].dst;
     HC_TRYCUDA(cudaMemcpyAsync(dst, d2h[i], bt->copies[i].bytes, cudaMemcpyDeviceToHost, st));
@@ -2066,6 +2113,7 @@ struct hc_plan {
   std::vector<void*> dev;
   cudaEvent_t ek0 = nullptr, ek1 = nullptr, ek2 = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;  // graph edges of the re-tracking branch
+  cudaEvent_t fork2 = nullptr, join2 = nullptr;  // and of the early re-tracking
   cudaEvent_t done = nullptr;  // recorded after each run's last copy
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -2077,7 +2125,7 @@ void free_plan(hc_plan* pl) {
   if (pl->graph) cudaGraphDestroy(pl->graph);
   if (pl->done) cudaEventSynchronize(pl->done);
   for (void* q : pl->dev) cudaFree(q);
-  for (cudaEvent_t e : {pl->ek0, pl->ek1, pl->ek2, pl->fork, pl->join, pl->done})
+  for (cudaEvent_t e : {pl->ek0, pl->ek1, pl->ek2, pl->fork, pl->join, pl->fork2, pl->join2, pl->done})
     if (e) cudaEventDestroy(e);
   pl->magic = 0;
   delete pl;
@@ -2144,7 +2192,7 @@ hc_status hc_plan_create(hc_problem* p, int32_t n_instances, hc_plan** out) {
   if ((rc = dalloc(sizeof(double) * items, &q)) != HC_OK) return fail(rc);
   pl->B.d_be = (double*)q;
   if ((rc = alloc_scratch(p, pl->n_inst, pl->B, dalloc)) != HC_OK) return fail(rc);
-  for (cudaEvent_t* e : {&pl->ek0, &pl->ek1, &pl->ek2, &pl->fork, &pl->join, &pl->done})
+  for (cudaEvent_t* e : {&pl->ek0, &pl->ek1, &pl->ek2, &pl->fork, &pl->join, &pl->fork2, &pl->join2, &pl->done})
     if (cudaEventCreate(e) != cudaSuccess) {
       set_err("cudaEventCreate failed");
       return fail(HC_ERR_CUDA);
@@ -2152,19 +2200,21 @@ hc_status hc_plan_create(hc_problem* p, int32_t n_instances, hc_plan** out) {
   // Capture on private streams (a shared stream could pick up another
   // thread's work while it is being captured); the re-tracking branch keeps
   // the high priority it has outside graphs.
-  cudaStream_t cap = nullptr, cap_hi = nullptr;
+  cudaStream_t cap = nullptr, cap_hi = nullptr, cap_hi2 = nullptr;
   int lo = 0, hi = 0;
   cudaDeviceGetStreamPriorityRange(&lo, &hi);
   if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaStreamCreateWithPriority(&cap_hi, cudaStreamNonBlocking, hi) != cudaSuccess) {
+      cudaStreamCreateWithPriority(&cap_hi, cudaStreamNonBlocking, hi) != cudaSuccess ||
+      cudaStreamCreateWithPriority(&cap_hi2, cudaStreamNonBlocking, hi) != cudaSuccess) {
     if (cap) cudaStreamDestroy(cap);
+    if (cap_hi) cudaStreamDestroy(cap_hi);
     set_err("cudaStreamCreate failed");
     return fail(HC_ERR_CUDA);
   }
   cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    const EnqEvents ev{pl->ek0, pl->ek1, pl->ek2, pl->fork, pl->join, true};
-    rc = enqueue_compute(p, pl->n_inst, pl->B, cap, cap_hi, ev);
+    const EnqEvents ev{pl->ek0, pl->ek1, pl->ek2, pl->fork, pl->join, pl->fork2, pl->join2, true};
+    rc = enqueue_compute(p, pl->n_inst, pl->B, cap, cap_hi, cap_hi2, ev);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(cap, &g);
     pl->graph = g;
@@ -2172,6 +2222,7 @@ hc_status hc_plan_create(hc_problem* p, int32_t n_instances, hc_plan** out) {
       e = cudaGraphInstantiateWithFlags(&pl->exec, pl->graph,
                                         cudaGraphInstantiateFlagUseNodePriority);
   }
+  cudaStreamDestroy(cap_hi2);
   cudaStreamDestroy(cap_hi);
   cudaStreamDestroy(cap);
   if (rc != HC_OK) return fail(rc);
@@ -2333,7 +2384,7 @@ hc_status hc_poll(hc_batch* b, int64_t timeout_us, hc_batch_result* r) {
     r->steps_accepted = (int64_t)s[5];
     r->steps_rejected = (int64_t)s[6];
     r->newton_iters = (int64_t)s[7];
-    r->escalated = (int64_t)b->h_ctl[2] + (int64_t)b->h_ctl[7];
+    r->escalated = (int64_t)b->h_ctl[2] + (int64_t)b->h_ctl[7] + (int64_t)b->h_ctl[20];
     r->esc_accepted = (int64_t)b->h_ctl[3];
     r->esc_rejected = (int64_t)b->h_ctl[4];
     r->esc_newton = (int64_t)b->h_ctl[5];
@@ -2519,7 +2570,7 @@ cudaError_t launch_dedupe(int64_t items, int64_t paths, int n, const float2* x32
   if (list) {
     const int grid = (int)std::min<int64_t>((items + 7) / 8, 1024);
     dedupe_list_kernel<<<std::max(grid, 1), 256, 0, st>>>(paths, n, x32, status, tol, list,
-                                                         list_count, out_list, out_count, t_io,
+                                                         list_count, out_list, 1, out_count, t_io,
                                                          1, nullptr);
   } else {
     return dedupe_all(items, paths, n, x32, status, tol, out_list, out_count, t_io, 1, nullptr,
@@ -2788,6 +2839,7 @@ void free_stream(hc_stream* s) {
 hc::LaunchCommon stream_common(const hc_stream* s) {
   hc::LaunchCommon c;
   std::memset(&c, 0, sizeof(c));
+  c.items_step = 1;
   c.s = dev_settings(s->p->s);
   c.paths = s->paths;
   return c;

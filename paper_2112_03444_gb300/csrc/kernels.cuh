@@ -85,8 +85,15 @@ struct LaunchCommon {
   uint8_t* status_out;                  // [items]
   int32_t* steps_out;                   // [items][3]
   double* be_out;                       // [items] (optional)
+  int items_step;                       // 1, or -1: items runs downwards
   int64_t* esc_list;                    // mixed precision: items to re-track in FP64
   unsigned long long* esc_count;
+  // Batches: items that have to wait for the duplicate check and the tier before
+  // (suspect conditions, that tier's own failures) go to this list instead, which
+  // runs downwards from late_end (the end of esc_list's array; together the two
+  // lists hold an item once).  nullptr: all to esc_list.
+  int64_t* late_end;
+  unsigned long long* late_count;
   // Hand-over between the FP32 and FP64 tiers:
   double* t_io;                 // per item: t to resume from in FP64 (0 = restart at t = 0)
   float2* x32_out;              // per item endpoint copy for duplicate detection (NaN if not finite)

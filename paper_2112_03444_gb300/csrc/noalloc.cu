@@ -295,6 +295,7 @@ extern "C" hc_status hc_track_dense_noalloc(int32_t n, int32_t degree, const dou
   std::memset(&a, 0, sizeof(a));
   a.c.s = hc::to_dev_settings(*settings);
   a.c.n_items = items;
+  a.c.items_step = 1;
   a.c.queue = ctl + 0;
   a.c.paths = paths;
   a.c.x_out = x_out;

@@ -524,8 +524,13 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
             const int64_t slot = RING ? item / c.paths : 0;
             const int64_t rec = RING ? item - slot * c.paths : item;
             if (to64) {
-              const unsigned long long pos = atomicAdd(c.esc_count + slot, 1ull);
-              c.esc_list[slot * c.paths + pos] = rec;
+              if (c.late_end && (base == ST_SINGULAR || c.start_hi)) {
+                const unsigned long long pos = atomicAdd(c.late_count, 1ull);
+                *(c.late_end - (int64_t)pos) = rec;
+              } else {
+                const unsigned long long pos = atomicAdd(c.esc_count + slot, 1ull);
+                c.esc_list[slot * c.paths + pos] = rec;
+              }
             } else {
               const unsigned long long pos = atomicAdd(c.dup_count + slot, 1ull);
               c.dup_list[slot * c.paths + pos] = rec;
@@ -663,7 +668,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         else
           break;
       } else {
-        if (!RING) item = c.items ? c.items[q] : (int64_t)q;
+        if (!RING) item = c.items ? c.items[(int64_t)q * c.items_step] : (int64_t)q;
         const int64_t inst = item / c.paths;
         inst_cur = inst;
         const int64_t k_in = item - inst * c.paths;
