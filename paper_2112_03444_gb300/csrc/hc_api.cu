@@ -410,6 +410,8 @@ struct hc_problem {
   hc::TermRec* d_rec = nullptr;
   double2* d_s64 = nullptr;
   hc::cdf* d_sdf = nullptr;  // the coefficients as double-floats
+  int32_t* d_sum_ptr[2] = {nullptr, nullptr};  // TermArgs sum_ptr, sum_ent
+  uint32_t* d_sum_ent[2] = {nullptr, nullptr};
   // coefficient interpolation: per (slot, row) the term's parameter factors
   // [TT][L][maxpf] (-1: none), and c(p0) in FP64 / FP32 / double-float
   bool coef_mode = false;
@@ -1019,6 +1021,28 @@ bool encode_terms(hc_problem* p, std::vector<hc::TermRec>& rec, std::vector<doub
   return true;
 }
 
+// The double-float kernels' summation lists (TermArgs sum_ptr, sum_ent) for paths
+// of `warps` warps, from the encoded records.
+void build_sums(const hc_problem* p, const std::vector<hc::TermRec>& rec, int warps,
+                std::vector<int32_t>& ptr, std::vector<uint32_t>& ent) {
+  const int n = p->n, L = p->L, NT = 32 * warps, CH = hc::term_df_slots(n, warps);
+  ptr.assign(1, 0);
+  ent.clear();
+  for (int k0 = 0; k0 < p->TT; k0 += CH)
+    for (int e = 0; e < n * n + n; ++e) {
+      const int i = e < n * n ? e % n : e - n * n, target = e < n * n ? e / n : n;
+      for (int kk = 0; kk < CH && k0 + kk < p->TT; ++kk) {
+        const hc::TermRec& r = rec[(size_t)(k0 + kk) * L + i];
+        for (int f = r.d - 1; f >= 0; --f)
+          if (r.tgt[f] == target)
+            ent.push_back((uint32_t)(f * NT + kk * n + i) |
+                          (target == n ? (uint32_t)(r.idx[f] + p->P) << 16 : 0u));
+      }
+      ptr.push_back((int32_t)ent.size());
+    }
+  ent.push_back(0);  // read ahead of the last entry's end
+}
+
 template <class T>
 hc_status upload(const std::vector<T>& v, T** out) {
   *out = nullptr;
@@ -1038,6 +1062,10 @@ void free_problem(hc_problem* p) {
   cudaFree(p->d_rec);
   cudaFree(p->d_s64);
   cudaFree(p->d_sdf);
+  for (int v = 0; v < 2; ++v) {
+    cudaFree(p->d_sum_ptr[v]);
+    cudaFree(p->d_sum_ent[v]);
+  }
   cudaFree(p->d_cpar);
   cudaFree(p->d_c0);
   cudaFree(p->d_c0f);
@@ -1358,6 +1386,10 @@ hc_status hc_create_problem(const hc_problem_desc* d, hc_problem** out) {
       set_err("this build has parameter-homotopy kernels for n <= 24");
       return HC_ERR_UNSUPPORTED;
     }
+    std::vector<int32_t> ptr[2];
+    std::vector<uint32_t> ent[2];
+    build_sums(p, rec, 1, ptr[0], ent[0]);
+    if (hc::term_df_warps(n) > 1) build_sums(p, rec, hc::term_df_warps(n), ptr[1], ent[1]);
     // double-float split of every coefficient: hi the nearest float, lo the
     // nearest float to the remainder
     std::vector<hc::cdf> sdf(s64.size());
@@ -1393,6 +1425,10 @@ hc_status hc_create_problem(const hc_problem_desc* d, hc_problem** out) {
     hc_status st;
     if ((st = upload(rec, &p->d_rec)) != HC_OK || (st = upload(s64, &p->d_s64)) != HC_OK ||
         (st = upload(sdf, &p->d_sdf)) != HC_OK || (st = upload(cpar, &p->d_cpar)) != HC_OK ||
+        (st = upload(ptr[0], &p->d_sum_ptr[0])) != HC_OK ||
+        (st = upload(ent[0], &p->d_sum_ent[0])) != HC_OK ||
+        (st = upload(ptr[1], &p->d_sum_ptr[1])) != HC_OK ||
+        (st = upload(ent[1], &p->d_sum_ent[1])) != HC_OK ||
         (st = upload(c0, &p->d_c0)) != HC_OK || (st = upload(c0f, &p->d_c0f)) != HC_OK ||
         (st = upload(c0df, &p->d_c0df)) != HC_OK ||
         (st = upload(p0v, &p->d_p0)) != HC_OK || (st = upload(sv, &p->d_start)) != HC_OK ||
@@ -1716,6 +1752,10 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
     ta.rec = p->d_rec;
     ta.s64 = p->d_s64;
     ta.sdf = p->d_sdf;
+    for (int v = 0; v < 2; ++v) {
+      ta.sum_ptr[v] = p->d_sum_ptr[v];
+      ta.sum_ent[v] = p->d_sum_ent[v];
+    }
     ta.TT = p->TT;
     ta.P = p->P;
     ta.ls = p->L;
@@ -2668,6 +2708,10 @@ extern "C" hc_status hc_evaluate(const hc_problem* p, int32_t precision, int32_t
       a.rec = p->d_rec;
       a.s64 = p->d_s64;
       a.sdf = p->d_sdf;
+      for (int v = 0; v < 2; ++v) {
+        a.sum_ptr[v] = p->d_sum_ptr[v];
+        a.sum_ent[v] = p->d_sum_ent[v];
+      }
       a.TT = p->TT;
       a.P = p->P;
       a.ls = p->L;
@@ -3007,6 +3051,10 @@ hc::TermArgs stream_term_args(const hc_stream* s, int64_t slot) {
   a.rec = p->d_rec;
   a.s64 = p->d_s64;
   a.sdf = p->d_sdf;
+  for (int v = 0; v < 2; ++v) {
+    a.sum_ptr[v] = p->d_sum_ptr[v];
+    a.sum_ent[v] = p->d_sum_ent[v];
+  }
   a.TT = p->TT;
   a.P = p->P;
   a.ls = p->L;

@@ -164,6 +164,13 @@ struct TermArgs {
   const TermRec* rec;    // [TT][ls]: term slot k of row i at k * ls + i
   const double2* s64;    // FP64 coefficients, same layout
   const cdf* sdf;        // the same as double-floats (mixed-precision residuals)
+  // Double-float kernels (term_block.cuh): which products every entry of the rows
+  // sums in a round of terms, for paths of one warp [0] and of several [1].
+  // Round c, entry e: sum_ent[sum_ptr[c (n n + n) + e] ..), e = i + n j for
+  // dH_i/dx_j, n n + i for dH_i/dt; an entry's low half is the product's place,
+  // its high half the position of the factor's dp in V (dH/dt).
+  const int32_t* sum_ptr[2];
+  const uint32_t* sum_ent[2];
   int TT;                // term slots per row (rows padded with zero terms)
   int P;                 // number of parameters
   int ls;                // lane stride of the tables (and V's offset of the 1)
@@ -183,6 +190,12 @@ struct TermArgs {
   const float2* dcf;
   const cdf* dcdf;
 };
+
+// Warps per path of the double-float term kernels (term_block.cuh): the terms of an
+// equation grow with n, and a round takes one per thread.
+__host__ __device__ constexpr int term_df_warps(int n) { return n <= 4 ? 1 : n <= 8 ? 2 : 4; }
+// Term slots per round of a path of `warps` warps
+__host__ __device__ constexpr int term_df_slots(int n, int warps) { return 32 * warps / n; }
 
 // Points at which hc_evaluate evaluates the homotopy (device buffers):
 // point k belongs to instance inst[k], lies at x[k] (n complex) and t[k];

@@ -16,12 +16,12 @@
 // commands (evaluate, residual, solve, exit).
 //
 // Measured against one row per lane (unrolled, 265 to 405 KB of code), ms: the
-// re-tracking tiers of trifocal (4 scenes, at most 800 steps) 600 -> 311, of 4-view
-// triangulation (600) 179 -> 101, of P3P (3000) 16.3 -> 12.4; precision DF on the
-// same (at most 300 steps) 1200 -> 523, 4471 -> 4284, 35 -> 26.  Warps per path: four
-// above 8 unknowns (trifocal tiers 774 / 470 / 326 / 319 with 1 / 2 / 4 / 8 warps,
-// precision DF 1478 / 714 / 583 / 753), one up to 4, where the items of a precision DF
-// batch fill the warps (P3P 33 / 55 / 85 with 1 / 2 / 4).
+// re-tracking tiers of trifocal (4 scenes, at most 800 steps) 600 -> 219, of 4-view
+// triangulation (600) 179 -> 85, of P3P (3000) 16.3 -> 7.0; precision DF on the
+// same (at most 300 steps) 1200 -> 413, 4471 -> 3321, 35 -> 20.  Warps per path: four
+// above 8 unknowns (before the summation lists, trifocal tiers 774 / 470 / 326 / 319
+// with 1 / 2 / 4 / 8 warps, precision DF 1478 / 714 / 583 / 753), one up to 4, where
+// the items of a precision DF batch fill the warps (P3P 33 / 55 / 85 with 1 / 2 / 4).
 #pragma once
 
 #include "kernels.cuh"
@@ -37,7 +37,7 @@ struct TermBlock {
   static constexpr int PP = 32 / LR, OWN = PP * NW;  // replicas per warp, per path
   static constexpr int PARTS = 1, ROWL = LR, WARPS = NW;
   static constexpr int NT = 32 * NW;   // threads of a path
-  static constexpr int CH = NT / N;    // term slots per round: one term per thread
+  static constexpr int CH = term_df_slots(N, NW);  // term slots per round: one term per thread
   static constexpr bool kCoop = false;
   enum : int { OP_EXIT = 0, OP_EVAL = 1, OP_RESIDUAL = 2, OP_SOLVE = 3 };
   struct Cmd {
@@ -174,49 +174,51 @@ struct TermBlock {
       }
       sync();
       // Every entry of the rows adds its products in the order of the terms,
-      // inside a term from the last factor to the first.  The long chains,
-      // dH_i/dt (every parameter factor) and H_i (every term), are the last
-      // entries, in a warp of their own.
-      constexpr int E0 = (N * N + 31) & ~31;
+      // inside a term from the last factor to the first, from the round's lists
+      // (trifocal, thousand cycles an evaluation: a search of the records 25, the
+      // lists 9, the products 8).  The long chains, dH_i/dt (every parameter factor) and H_i
+      // (every term), are the last entries, in a warp of their own.
+      constexpr int E0 = (N * N + 31) & ~31, E = N * N + N;
+      const int32_t* ptr = a->sum_ptr[NW > 1] + (int64_t)(k0 / CH) * E;
+      const uint32_t* ent = a->sum_ent[NW > 1];
 #pragma unroll 1
       for (int e = id; e < E0 + N; e += NT) {
         if (e >= N * N && e < E0) continue;
-        const int q = e < E0 ? e / N : N;
-        const int i = e < E0 ? e - q * N : e - E0;
-        if (q < N) {
+        if (e < N * N) {
+          const int q = e / N, i = e - q * N;
+          int m = ptr[e];
+          const int end = ptr[e + 1];
+          if (m == end) continue;
           cx<df> v = M[q * LR + i];
-          const unsigned jj = (unsigned)q * 0x01010101u;
+          uint32_t w = ent[m];
 #pragma unroll 1
-          for (int kk = 0; kk < nk; ++kk) {
-            const cx<df>* c = C() + kk * N + i;
-            const uint2 tg = *reinterpret_cast<const uint2*>((a->rec + (int64_t)(k0 + kk) * LS + i)->tgt);
-            unsigned long long hit =
-                (unsigned long long)__vcmpeq4(tg.y, jj) << 32 | __vcmpeq4(tg.x, jj);
-            while (hit != 0) {
-              const int f = 7 - (__clzll((long long)hit) >> 3);
-              hit &= ~(0xffull << (8 * f));
-              v = v + c[f * NT];
-            }
+          while (m < end) {
+            const uint32_t next = ent[++m];  // (one entry of padding behind the last)
+            v = v + C()[w & 0xffffu];
+            w = next;
           }
           M[q * LR + i] = v;
           continue;
         }
+        const int i = e - E0;
         if (want & WANT_HT) {
           cx<df> v = M[N * LR + i];
+          if (a->coef_mode) {
 #pragma unroll 1
-          for (int kk = 0; kk < nk; ++kk) {
-            const int64_t r = (int64_t)(k0 + kk) * LS + i;
-            const cx<df>* c = C() + kk * N + i;
-            const unsigned long long idx = *reinterpret_cast<const unsigned long long*>(a->rec[r].idx);
-            const unsigned long long tgt = *reinterpret_cast<const unsigned long long*>(a->rec[r].tgt);
-#pragma unroll 1
-            for (int f = a->rec[r].d - 1; f >= 0; --f)
-              if (((int)(tgt >> (8 * f)) & 255) == N)
-                v = cfma(c[f * NT], Vx[((int)(idx >> (8 * f)) & 255) + P], v);
-            if (a->coef_mode) {
+            for (int kk = 0; kk < nk; ++kk) {
               cx<df> s, dcr;
-              coef(r, t, s, dcr);
-              v = cfma(dcr, c[kMaxTermFactors * NT], v);
+              coef((int64_t)(k0 + kk) * LS + i, t, s, dcr);
+              v = cfma(dcr, C()[kMaxTermFactors * NT + kk * N + i], v);
+            }
+          } else {
+            int m = ptr[N * N + i];
+            const int end = ptr[N * N + i + 1];
+            uint32_t w = ent[m];
+#pragma unroll 1
+            while (m < end) {
+              const uint32_t next = ent[++m];
+              v = cfma(C()[w & 0xffffu], Vx[w >> 16], v);
+              w = next;
             }
           }
           M[N * LR + i] = v;
@@ -311,13 +313,15 @@ struct TermBlock {
   }
 
   // Gauss-Jordan as gj_solve_df on the first W columns: replica o of the rows
-  // (OWN in all) updates the columns j with j mod OWN = o.  The warp that holds
-  // column k + 1 updates it first, searches its pivot and publishes row and
-  // reciprocal (the longest chain of a pivot step) before its other columns,
-  // while the other warps are still at theirs: one barrier per pivot.  The pivot
-  // row's entries are read where they lie.  Returns whether every pivot was
-  // nonzero and finite; the lanes of the first replica hold 1 / pivot of their
-  // row and the column it pivoted on (-1: none).
+  // (OWN in all) updates the columns j with j mod OWN = o, which no other replica
+  // reads before they are pivot columns.  The warp that holds column k + 1 updates
+  // it first, searches its pivot and publishes row and reciprocal (the longest
+  // chain of a pivot step), and comes to its other columns behind the barrier,
+  // when the next column's warp is already at its search: one barrier per pivot
+  // (n = 18 with 4 warps: 22.3 -> 21.5 thousand cycles a solve).  The pivot row's
+  // entries are read where they lie.  Returns whether every pivot was nonzero and
+  // finite; the lanes of the first replica hold 1 / pivot of their row and the
+  // column it pivoted on (-1: none).
   struct Pivot {
     cx<df> inv;
     unsigned key;
@@ -361,7 +365,8 @@ struct TermBlock {
       const cx<df> l = me ? czero<df>() : M[LR * k + r] * inv;
       const cx<df> lr = neg(re_re(l)), li = neg(nim_im(l));
       int j = k + 1 + ((own - (k + 1)) & (OWN - 1));  // this lane's first column
-      if (k + 1 < N && ((k + 1) & (OWN - 1)) / PP == w) {
+      const bool ahead = k + 1 < N && ((k + 1) & (OWN - 1)) / PP == w;
+      if (ahead) {
         const bool first = j == k + 1;
         cx<df> v = czero<df>();
         if (first) {
@@ -373,6 +378,7 @@ struct TermBlock {
         __syncwarp();
         search(k + 1);
         if (first) j += OWN;
+        sync();
       }
 #pragma unroll 1
       for (; __any_sync(0xffffffffu, j < W); j += UNROLL * OWN) {
@@ -388,7 +394,7 @@ struct TermBlock {
         for (int u = 0; u < UNROLL; ++u)
           if (j + u * OWN < W) M[LR * (j + u * OWN) + r] = v[u];
       }
-      sync();
+      if (!ahead) sync();
     }
     if (g.wl >= LR || r >= N) col = -1;
     return (lo & ~31u) != 0u && (hi & ~31u) < 0x7f800000u;

@@ -7,15 +7,12 @@
 
 namespace hc {
 
-// Two warps for up to 8 unknowns, four above: the terms of an equation grow
-// with n, and a round takes one per thread.
 template <int N>
 KernelRef pick_term_df(int n, int lanes) {
   if constexpr (N == 0) {
     return KernelRef{nullptr, 0};
   } else {
-    constexpr int NW = N <= 4 ? 1 : N <= 8 ? 2 : 4;
-    if (n == N) return lanes == 32 ? term_df_ref<N, 1>() : term_df_ref<N, NW>();
+    if (n == N) return lanes == 32 ? term_df_ref<N, 1>() : term_df_ref<N, term_df_warps(N)>();
     return pick_term_df<N - 1>(n, lanes);
   }
 }
