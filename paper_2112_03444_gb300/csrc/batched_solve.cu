@@ -138,11 +138,14 @@ SolveRef solve_ref(int dev) {
   SolveRef k{reinterpret_cast<const void*>(&batched_solve_kernel<N, R, D>),
              solve_smem_bytes<N, R, D>(), kThreads / solve_lanes<N, D>(),
              dev < kMaxDevices ? known[dev].load(std::memory_order_acquire) : 0};
-  if (k.per_sm > 0) return k;
+  // (the attribute belongs to the context, which a program may have replaced)
   if (k.smem > 48 * 1024 &&
       cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) !=
-          cudaSuccess)
+          cudaSuccess) {
+    k.per_sm = 0;
     return k;
+  }
+  if (k.per_sm > 0) return k;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k.per_sm, k.fn, kThreads, k.smem) !=
       cudaSuccess)
     k.per_sm = 0;
