@@ -49,7 +49,12 @@ constexpr int kTrackMinBlocks = 4;
 // HC_PREC_FP64, or HC_PREC_DF (FP64 state, double-float evaluation and
 // solve).  The double-float kernels hold every complex number in four
 // registers and run one path per warp: they get the registers of one block
-// per SM rather than of four.
+// per SM rather than of four (142 at quadratic n = 12, 152 at cubic n = 8).
+// What bounds them is the latency of a path, so spills cost more than warps
+// give: compiled for 4 / 5 blocks, re-tracking of cubic n = 8 (16 systems)
+// 13.3 -> 14.5 / 21.0 ms, precision DF on it 433 -> 419 / 448 ms.  Two or four
+// warps per path (columns over the warps) lose as well: re-tracking 13.2 / 11.6
+// ms, precision DF 782 / 1070 ms.
 template <int N, int DEG, int PREC, int L, bool RING = false>
 __global__ void __launch_bounds__(kBlock, PREC == HC_PREC_DF ? 1 : kTrackMinBlocks)
     dense_td_kernel(const DenseArgs a) {

@@ -65,7 +65,6 @@ __device__ __forceinline__ df to_df(double v) {
 }
 __device__ __forceinline__ float df_to_float(df a) { return __fadd_rn(a.hi, a.lo); }
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ df df_neg(df a) { return df{-a.hi, -a.lo}; }
 
 // c + x1 y1 + x2 y2.  The two leading products are exact (TwoProd); their
 // errors and the cross terms hi * lo go into the low part (the dropped

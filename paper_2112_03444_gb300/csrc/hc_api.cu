@@ -1684,7 +1684,7 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
   // them on hs2; the others (from the end of esc_list, ctl[20]) behind that
   // tier.  Measured, re-tracking time in ms: trifocal (4 scenes, at most 800 steps)
   // 327 -> 266, cubic n = 8 (16 systems) 17.5 -> 13.3, P3P (3000) 12.4 -> 9.6, quadratic
-  // n = 12 (16) 4.7 -> 3.1.
+  // n = 12 (16) 4.7 -> 3.1 (trifocal now 219 and P3P 7.0: term_block.cuh).
   hc::LaunchCommon cd = cm;
   cd.count_dev = B.d_ctl + 7;
   cd.items = B.dup_list;
