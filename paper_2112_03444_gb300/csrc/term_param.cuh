@@ -320,7 +320,7 @@ template <int N, int PREC, int L, bool RING = false>
 __global__ void __launch_bounds__(kBlock) term_param_kernel(const __grid_constant__ TermArgs a) {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L, groups_meet(L, RING)>();
+  const Group g = make_group<L, groups_meet(L, RING, MIXED)>();
   const GroupMem sm = make_group_mem<L>(smem, a.extra, term_acc_bytes<N, MIXED, L>(),
                                         endgame_smem_bytes(L, MIXED));
   TermProblem<N, L, MIXED> prob{&a, g, sm};

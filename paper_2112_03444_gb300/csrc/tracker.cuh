@@ -81,7 +81,14 @@ enum : int { M_RK = 0, M_NEWTON = 1, M_REFINE = 2, M_COND = 3, M_DONE = 4, M_FET
 
 // Kernels whose warps hold several groups and keep them in step (see
 // make_group); the groups of a resident launch wait for work on their own.
-__host__ __device__ constexpr bool groups_meet(int L, bool ring) { return !ring && L < 32; }
+// The all-FP64 kernels meet with two groups per warp only: an FP64 instruction
+// holds its pipe as long for one group as for all, and with four or eight groups
+// waiting for the slowest costs more than their separate instructions (ms, apart /
+// meeting: quadratic n = 6, 64 systems, 14.4 / 14.8; cubic n = 5, 24 systems, 29.3 /
+// 30.6; quadratic n = 12, 16 systems, two groups, 802 / 797).
+__host__ __device__ constexpr bool groups_meet(int L, bool ring, bool mixed) {
+  return !ring && L < 32 && (mixed || L == 16);
+}
 
 // Phases of the mixed kernels: the whole path in one loop (resident launches),
 // its FP32 phase only, or everything after it.
@@ -256,7 +263,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
   // Warps with several groups meet once per iteration and leave together (a
   // group out of work is M_IDLE until then): without that point the groups
   // drift apart and each runs the evaluation and the solve on its own.
-  constexpr bool MEET = groups_meet(L, RING);
+  constexpr bool MEET = groups_meet(L, RING, MIXED);
   constexpr int EP = COOP_EVAL ? 32 / L : 1;
   constexpr int GL = L * HOM::WARPS;  // threads of a path
   const DevSettings& s = c.s;
@@ -1116,7 +1123,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
 template <int N, int L, bool MIXED, class PROB, class RE = double, bool RING = false>
 __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon& c,
                                             const Group& g, const GroupMem& sm) {
-  if constexpr (MIXED && groups_meet(L, RING)) {
+  if constexpr (MIXED && groups_meet(L, RING, MIXED)) {
     if (!c.start_hi) {
       if (threadIdx.x == 0) *sm.hand = 0;
       __syncthreads();
