@@ -64,12 +64,17 @@ constexpr size_t solve_smem_bytes() {
                           (size_t)G * N);
 }
 
+// Blocks per SM to compile for (0: as the registers fall).  n = 8 in FP64 by six
+// registers misses the fifth block, which a batch of five blocks per SM needs.
 template <int N, class R, int D>
-__global__ void __launch_bounds__(kThreads) batched_solve_kernel(int64_t batch,
-                                                                 const cx<R>* __restrict__ A,
-                                                                 const cx<R>* __restrict__ b,
-                                                                 cx<R>* __restrict__ x,
-                                                                 int32_t* __restrict__ info) {
+constexpr int min_blocks() {
+  return sizeof(R) == 8 && D == 1 && N == 8 ? 5 : 0;
+}
+
+template <int N, class R, int D>
+__global__ void __launch_bounds__(kThreads, min_blocks<N, R, D>())
+    batched_solve_kernel(int64_t batch, const cx<R>* __restrict__ A, const cx<R>* __restrict__ b,
+                         cx<R>* __restrict__ x, int32_t* __restrict__ info) {
   constexpr int L = solve_lanes<N, D>(), G = kThreads / L, W = N + 1;
   constexpr int ROWS = (N + L - 1) / L;
   constexpr int S = (N + 2) & ~1;
@@ -92,33 +97,44 @@ __global__ void __launch_bounds__(kThreads) batched_solve_kernel(int64_t batch,
     const cx<R>* bb = b + base * N;
     for (int idx = threadIdx.x; idx < cnt * N; idx += kThreads) stage[idx * W + N] = bb[idx];
     __syncthreads();
-    cx<R> a[ROWS][W];
+    // FP64: a warp without a system solves nothing.  In one with some, the groups
+    // past the count take its last system again and the lanes past the last row ones:
+    // their results go nowhere, but a reciprocal of zero takes the division's slow
+    // path for the whole warp.  (us, with all groups of a block on zero rows -> now,
+    // n = 9: batch 1000 19.6 -> 17.7, one system more than a block per SM 30.5 -> 20.0.
+    // FP32 is bound by issue slots and pays more for the branch than for the rows.)
+    constexpr bool FILL = sizeof(R) == 8;
     const bool live = grp < cnt;
+    const bool work = !FILL || (threadIdx.x & ~31) / L < cnt;
+    const int sys = FILL && !live ? cnt - 1 : grp;
+    cx<R> a[ROWS][W];
 #pragma unroll
     for (int q = 0; q < ROWS; ++q)
 #pragma unroll
       for (int j = 0; j < W; ++j)
-        a[q][j] = (live && g.gl + q * L < N) ? stage[(grp * N + g.gl + q * L) * W + j]
-                                             : hc::czero<R>();
+        a[q][j] = (FILL || live) && g.gl + q * L < N ? stage[(sys * N + g.gl + q * L) * W + j]
+                                                     : hc::mk<R>(R(FILL ? 1 : 0), R(0));
     __syncthreads();  // the stage is free for the next round once every row is in registers
-    cx<R> sol[ROWS];
-    int col[ROWS];
-    bool ok;
-    if constexpr (ROWS == 1)
-      ok = hc::gj_solve<N, 1, R, L, true>(g, a[0], sol, col[0], pv);
-    else
-      ok = hc::gj_solve_rows<N, L, ROWS, R>(g, a, sol, col, pv);
-#pragma unroll
-    for (int q = 0; q < ROWS; ++q)
-      if (col[q] >= 0) sb[col[q]] = sol[q];
-    __syncwarp();
-    if (live) {
+    if (work) {
+      cx<R> sol[ROWS];
+      int col[ROWS];
+      bool ok;
+      if constexpr (ROWS == 1)
+        ok = hc::gj_solve<N, 1, R, L, true>(g, a[0], sol, col[0], pv);
+      else
+        ok = hc::gj_solve_rows<N, L, ROWS, R>(g, a, sol, col, pv);
 #pragma unroll
       for (int q = 0; q < ROWS; ++q)
-        if (g.gl + q * L < N) x[(base + grp) * N + g.gl + q * L] = sb[g.gl + q * L];
-      if (g.gl == 0 && info) info[base + grp] = ok ? 0 : 1;
+        if (col[q] >= 0) sb[col[q]] = sol[q];
+      __syncwarp();
+      if (live) {
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q)
+          if (g.gl + q * L < N) x[(base + grp) * N + g.gl + q * L] = sb[g.gl + q * L];
+        if (g.gl == 0 && info) info[base + grp] = ok ? 0 : 1;
+      }
+      __syncwarp();
     }
-    __syncwarp();
   }
 }
 
