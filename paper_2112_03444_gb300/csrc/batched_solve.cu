@@ -71,18 +71,21 @@ constexpr int min_blocks() {
   return sizeof(R) == 8 && D == 1 && N == 8 ? 5 : 0;
 }
 
-template <int N, class R, int D>
+// MEET: the groups of a warp in step; otherwise each group runs by itself and those
+// past the batch not at all (a few FP32 systems, see solve_dispatch).
+template <int N, class R, int D, bool MEET>
 __global__ void __launch_bounds__(kThreads, min_blocks<N, R, D>())
     batched_solve_kernel(int64_t batch, const cx<R>* __restrict__ A, const cx<R>* __restrict__ b,
                          cx<R>* __restrict__ x, int32_t* __restrict__ info) {
   constexpr int L = solve_lanes<N, D>(), G = kThreads / L, W = N + 1;
   constexpr int ROWS = (N + L - 1) / L;
   constexpr int S = (N + 2) & ~1;
+  static_assert(MEET || ROWS == 1, "groups apart: one row per lane");
   extern __shared__ __align__(16) unsigned char smem[];
   cx<R>* stage = reinterpret_cast<cx<R>*>(smem);
   cx<R>* pvbuf = stage + (((size_t)G * N * W + 1) & ~(size_t)1);
   cx<R>* sbuf = pvbuf + (size_t)G * 2 * S;
-  const hc::Group g = hc::make_group<L, true>();
+  const hc::Group g = hc::make_group<L, MEET>();
   const int grp = threadIdx.x / L;
   cx<R>* pv = pvbuf + grp * 2 * S;
   cx<R>* sb = sbuf + grp * N;
@@ -105,7 +108,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks<N, R, D>())
     // FP32 is bound by issue slots and pays more for the branch than for the rows.)
     constexpr bool FILL = sizeof(R) == 8;
     const bool live = grp < cnt;
-    const bool work = !FILL || (threadIdx.x & ~31) / L < cnt;
+    const bool work = MEET ? !FILL || (threadIdx.x & ~31) / L < cnt : live;
     const int sys = FILL && !live ? cnt - 1 : grp;
     cx<R> a[ROWS][W];
 #pragma unroll
@@ -120,20 +123,20 @@ __global__ void __launch_bounds__(kThreads, min_blocks<N, R, D>())
       int col[ROWS];
       bool ok;
       if constexpr (ROWS == 1)
-        ok = hc::gj_solve<N, 1, R, L, true>(g, a[0], sol, col[0], pv);
+        ok = hc::gj_solve<N, 1, R, L, MEET>(g, a[0], sol, col[0], pv);
       else
         ok = hc::gj_solve_rows<N, L, ROWS, R>(g, a, sol, col, pv);
 #pragma unroll
       for (int q = 0; q < ROWS; ++q)
         if (col[q] >= 0) sb[col[q]] = sol[q];
-      __syncwarp();
+      __syncwarp(g.meet);
       if (live) {
 #pragma unroll
         for (int q = 0; q < ROWS; ++q)
           if (g.gl + q * L < N) x[(base + grp) * N + g.gl + q * L] = sb[g.gl + q * L];
         if (g.gl == 0 && info) info[base + grp] = ok ? 0 : 1;
       }
-      __syncwarp();
+      __syncwarp(g.meet);
     }
   }
 }
@@ -148,10 +151,10 @@ struct SolveRef {
 
 // The occupancy query costs as much as the launch of a small batch: once per
 // kernel and device.
-template <int N, class R, int D>
+template <int N, class R, int D, bool MEET = true>
 SolveRef solve_ref(int dev) {
   static std::atomic<int> known[kMaxDevices];
-  SolveRef k{reinterpret_cast<const void*>(&batched_solve_kernel<N, R, D>),
+  SolveRef k{reinterpret_cast<const void*>(&batched_solve_kernel<N, R, D, MEET>),
              solve_smem_bytes<N, R, D>(), kThreads / solve_lanes<N, D>(),
              dev < kMaxDevices ? known[dev].load(std::memory_order_acquire) : 0};
   // (the attribute belongs to the context, which a program may have replaced)
@@ -180,6 +183,12 @@ SolveRef solve_dispatch(int n, int64_t batch, int sms, int dev) {
       constexpr int D = wide_rows<N, R>();
       if (D > 1 && batch >= (int64_t)kFillWarps * sms * (32 / solve_lanes<N, 1>()))
         return solve_ref<N, R, D>(dev);
+      // A few FP32 systems: the group-wide maximum of one group is faster than the
+      // butterfly that several share, and the other warps stay out of the way (one
+      // system, device us, in step / apart: n = 8 2.8 / 2.6, n = 16 4.2 / 3.7, n = 32
+      // 7.9 / 7.4; two systems: n = 8 2.8 / 3.2, n = 16 4.1 / 4.8, n = 32 8.2 / 7.9).
+      if constexpr (sizeof(R) == 4)
+        if (batch < (solve_lanes<N, 1>() == 32 ? 4 : 2)) return solve_ref<N, R, 1, false>(dev);
       return solve_ref<N, R, 1>(dev);
     }
     return solve_dispatch<R, N + 1>(n, batch, sms, dev);

@@ -90,3 +90,13 @@ def test_ragged_last_block(env, n, dtype):
     err = np.abs(x[1:].to(wide).cpu().numpy() - want).max(1) / np.abs(want).max(1)
     u = 2.0 ** -24 if dtype == "complex64" else 2.0 ** -53
     assert (err <= 64 * n * np.linalg.cond(A64) * u).all()
+
+
+@pytest.mark.parametrize("n", [8, 13, 16])
+def test_one_fp32_system_is_no_slower_than_two(env, n):
+    """One system has no company to keep in step with: the maximum over its own
+    lanes, not the butterfly that the groups of a warp share."""
+    torch, _ = env
+    t1 = _device_us(env, n, 1, torch.complex64)
+    t2 = _device_us(env, n, 2, torch.complex64)
+    assert t1 <= 0.97 * t2, (t1, t2)
