@@ -39,19 +39,50 @@ constexpr int kThreads = 128;
 // rows per lane a warp's reciprocals serve D times the systems: batch 100,000, us,
 // one row -> D rows: n = 5 289 -> 141, n = 8 494 -> 361, n = 12 1763 -> 977 (D = 4),
 // n = 13 1981 -> 1594, n = 20 7550 -> 6475 (D = 2; four rows of 13 or more entries
-// leave the registers).  A batch that does not fill the chip is bound by latency,
-// which the rows per lane lengthen (n = 13, batch 1000: 33 -> 46), so they are used
-// from 16 one-row warps per SM on: the two cross between 8 (n = 13, 20) and 14 (n = 4,
-// 8).  FP32 is bound by issue slots and its row updates: one row per lane (n = 20,
-// batch 100,000: 281 against 343 with two rows and two-wide updates).
+// leave the registers).  Where they pay is decided by several_rows.  FP32 is bound
+// by issue slots and its row updates: one row per lane (n = 20, batch 100,000: 281
+// against 343 with two rows and two-wide updates).
 template <int N, class R>
 constexpr int wide_rows() {
   return sizeof(R) == 4 || N > 24 ? 1 : N > 12 || N <= 2 ? 2 : 4;
 }
-constexpr int kFillWarps = 16;  // one-row warps per SM from which on
 template <int N, int D>
 constexpr int solve_lanes() {
   return (N <= 4 ? 4 : N <= 8 ? 8 : N <= 16 ? 16 : 32) / D;
+}
+
+// A block of D rows per lane holds D times the systems and takes longer, so what
+// counts is how many rounds (blocks on the busiest SM) either form needs: 6 rounds of
+// one-row blocks at n = 20 take 265 us, the 3 rounds of two-row blocks that hold the
+// same systems 316 (the hardware gives some SM a fourth).  round_cost: a round of
+// D-row blocks in percent of a round of one-row blocks, fitted to 60 batches of 1 to
+// 34 rounds at every n; the sizes that fill their lanes (4, 8, 16) and n = 7 have the
+// cheaper one-row rounds.  A third of a round is the wide form's longer latency.
+constexpr int round_cost(int n) {
+  return n <= 2                     ? 130
+         : n == 4 || n == 7 || n == 8 ? 265
+         : n <= 12                    ? 200
+         : n <= 15                    ? 150
+         : n <= 16                    ? 160
+         : n <= 20                    ? 165
+                                      : 175;
+}
+// Against one row per lane everywhere (us, one row / rule): n = 8, batch 9,728 48 / 39,
+// n = 10, 3,648 49 / 41, n = 20, 2,432 178 / 161; where the other form is taken: n = 20,
+// 3,648 265 (D rows 316), n = 24, 3,648 354 (D rows 435).
+template <int N, class R>
+bool several_rows(int64_t batch, int sms) {
+  constexpr int D = wide_rows<N, R>();
+  if constexpr (D == 1) return false;
+  const int64_t one = kThreads / solve_lanes<N, 1>(), wide = kThreads / solve_lanes<N, D>();
+  // (a last one-row block that is half empty costs half a round)
+  const int64_t r1 = (batch - one / 2 + one * sms - 1) / (one * sms);
+  const int64_t blocks = (batch + wide - 1) / wide;
+  int64_t r = (blocks + sms - 1) / sms;
+  // an odd round that is nearly full: the blocks beyond an even number per SM are not
+  // spread evenly, and some SM gets two of them
+  if (r > 2 && r % 2 == 1 && 10 * (r * sms - blocks) < 3 * sms) ++r;
+  return 100 * r1 > round_cost(N) * r + 35;
 }
 
 // Shared memory of one block: the staged augmented matrices [G][N][N + 1],
@@ -180,9 +211,7 @@ SolveRef solve_dispatch(int n, int64_t batch, int sms, int dev) {
     return SolveRef{nullptr, 0, 0, 0};
   } else {
     if (n == N) {
-      constexpr int D = wide_rows<N, R>();
-      if (D > 1 && batch >= (int64_t)kFillWarps * sms * (32 / solve_lanes<N, 1>()))
-        return solve_ref<N, R, D>(dev);
+      if (several_rows<N, R>(batch, sms)) return solve_ref<N, R, wide_rows<N, R>()>(dev);
       // A few FP32 systems: the group-wide maximum of one group is faster than the
       // butterfly that several share, and the other warps stay out of the way (one
       // system, device us, in step / apart: n = 8 2.8 / 2.6, n = 16 4.2 / 3.7, n = 32

@@ -100,3 +100,29 @@ def test_one_fp32_system_is_no_slower_than_two(env, n):
     t1 = _device_us(env, n, 1, torch.complex64)
     t2 = _device_us(env, n, 2, torch.complex64)
     assert t1 <= 0.97 * t2, (t1, t2)
+
+
+@pytest.mark.parametrize("n", [20, 24])
+def test_six_rounds_of_blocks(env, n):
+    """Six blocks per SM, three with two rows per lane (of which some SM would get
+    four): half again as long as four blocks per SM, and a fifth for the rounds."""
+    torch, _ = env
+    per_round = _per_block(n) * torch.cuda.get_device_properties(0).multi_processor_count
+    t4 = _device_us(env, n, 4 * per_round, torch.complex128)
+    t6 = _device_us(env, n, 6 * per_round, torch.complex128)
+    assert t6 <= 1.8 * t4, (t4, t6)
+
+
+@pytest.mark.parametrize("n", [2, 4, 8, 12, 16, 20, 24])
+def test_same_bits_on_both_sides_of_the_choice(env, n):
+    """Batches of 1 to 9 rounds take one row per lane or several: the same bits."""
+    torch, hc = env
+    per_round = _per_block(n) * torch.cuda.get_device_properties(0).multi_processor_count
+    A, b, x, info = _systems(torch, n, 9 * per_round, torch.complex128)
+    assert hc.batched_solve(A, b, x, info) == hc.HC_OK
+    for batch in [per_round * r + k for r in range(1, 9) for k in (-1, 0, 1, per_round // 2)]:
+        xs = torch.zeros_like(b[:batch])
+        infos = torch.full((batch,), 7, dtype=torch.int32, device="cuda")
+        assert hc.batched_solve(A[:batch], b[:batch], xs, infos) == hc.HC_OK
+        assert torch.equal(torch.view_as_real(xs), torch.view_as_real(x[:batch])), batch
+        assert torch.equal(infos, info[:batch]), batch
