@@ -385,7 +385,8 @@ struct TermBlock {
         cx<df> v[UNROLL];
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u) {
-          const int ju = LR * min(j + u * OWN, W - 1);
+          // (behind the last column: column k, which nobody writes now)
+          const int ju = LR * (j + u * OWN < W ? j + u * OWN : k);
           const cx<df> p = M[ju + rp];
           v[u] = dot2p(M[ju + r], lr, p, li, im_re(p));
         }
@@ -394,7 +395,12 @@ struct TermBlock {
         for (int u = 0; u < UNROLL; ++u)
           if (j + u * OWN < W) M[LR * (j + u * OWN) + r] = v[u];
       }
-      if (!ahead) sync();
+      // the next step's lanes read other lanes' entries of these columns (a vote
+      // orders no memory)
+      if (ahead)
+        __syncwarp();
+      else
+        sync();
     }
     if (g.wl >= LR || r >= N) col = -1;
     return (lo & ~31u) != 0u && (hi & ~31u) < 0x7f800000u;
