@@ -132,6 +132,7 @@ __device__ __forceinline__ unsigned long long hand_pop(const LaunchCommon& c,
                                                        unsigned long long* head) {
   unsigned long long h = *reinterpret_cast<volatile unsigned long long*>(head);
   while (h != 0) {
+    __threadfence_block();  // the link is read behind the head that published it
     const unsigned long long next = __ldcg(c.hand_list + hand_item(h));
     const unsigned long long was = atomicCAS(head, h, next);
     if (was == h) break;
@@ -610,6 +611,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         // after it (see run_tracker)
         unsigned long long e = 0;
         if (g.gl == 0) e = hand_pop(c, sm.hand);
+        __syncwarp(g.mask);  // every lane's reads of the item's slots come behind the pop
         e = __shfl_sync(g.mask, e, leader);
         if (e == 0) {
           if constexpr (MEET)

@@ -32,7 +32,15 @@
 
 namespace lanes {
 
-using Clock = std::vector<uint32_t>;
+constexpr int kMost = 128;  // threads of a block
+struct Clock {
+  uint32_t at[kMost];
+  LANES_RAW Clock() {
+    for (uint32_t& v : at) v = 0;
+  }
+  LANES_RAW uint32_t& operator[](int k) { return at[k]; }
+  LANES_RAW const uint32_t& operator[](int k) const { return at[k]; }
+};
 
 struct Thread {
   ucontext_t ctx;
@@ -45,18 +53,28 @@ struct Thread {
   Clock vc, released, pending;
 };
 
-struct Word {  // per 4 bytes of a watched range
+struct Word {
   int writer = -1;
   uint32_t at = 0;
-  std::map<int, uint32_t> reads;
+  bool read = false;
+  Clock reads;
+};
+struct Range {  // shared data, checked by words of `grain` bytes
+  uintptr_t begin;
+  size_t bytes, grain;
+  std::vector<Word> words;
+  Word* table;
 };
 
 struct Machine {
-  std::vector<Thread> th;
+  Thread* threads = nullptr;
+  int count = 0;
+  uint32_t joint[kMost];
+  Range* ranges = nullptr;
+  int range_count = 0;
   ucontext_t main;
   int cur = -1;
-  std::map<uintptr_t, size_t> watched;  // begin -> bytes
-  std::map<uintptr_t, Word> words;
+  std::vector<Range> watched;
   std::map<uintptr_t, Clock> atomics;   // words accessed by atomics: their clocks
   std::set<std::string> races;
   std::function<void()> body;
@@ -64,47 +82,54 @@ struct Machine {
 inline Machine* machine = new Machine;
 inline bool checking = false;  // the containers used by a check are instrumented too
 LANES_RAW inline Machine& m() { return *machine; }
-LANES_RAW inline Thread& me() { return m().th[m().cur]; }
+LANES_RAW inline Thread& me() { return m().threads[m().cur]; }
 
 LANES_RAW inline void join(Clock& a, const Clock& b) {
-  for (size_t k = 0; k < a.size(); ++k) a[k] = std::max(a[k], b[k]);
+  for (int k = 0; k < kMost; ++k) a[k] = a[k] > b[k] ? a[k] : b[k];
 }
 
-// An access of the running thread.
 LANES_RAW inline void check(const void* p, size_t bytes, bool write) {
   Machine& M = m();
   const uintptr_t a = (uintptr_t)p;
-  auto it = M.watched.upper_bound(a);
-  if (it == M.watched.begin()) return;
-  --it;
-  if (a >= it->first + it->second) return;
-  if (a + bytes > it->first + it->second) M.races.insert("access past the end of a buffer");
+  Range* r = nullptr;
+  for (int k = 0; k < M.range_count; ++k)
+    if (a - M.ranges[k].begin < M.ranges[k].bytes) r = M.ranges + k;
+  if (!r) return;
+  if (a + bytes > r->begin + r->bytes) {
+    M.races.insert("access past the end of a buffer");
+    return;
+  }
   Thread& t = me();
-  if (auto at = M.atomics.find(a); at != M.atomics.end()) {
+  auto at = M.atomics.find(a);
+  if (at != M.atomics.end()) {
     join(t.pending, at->second);
     return;
   }
-  for (uintptr_t w = a & ~(uintptr_t)3; w < a + bytes; w += 4) {
-    Word& x = M.words[w];
-    char msg[160];
+  for (size_t w = (a - r->begin) / r->grain; w * r->grain < a + bytes - r->begin; ++w) {
+    Word& x = r->table[w];
     auto race = [&](const char* what, int other) {
-      std::snprintf(msg, sizeof msg, "%s of thread %d, not ordered with a %s of thread %d, offset %zu",
-                    write ? "write" : "read", M.cur, what, other, (size_t)(w - it->first));
+      char msg[160];
+      std::snprintf(msg, sizeof msg,
+                    "buffer %d, offset %zu: %s of thread %d, not ordered with a %s of thread %d",
+                    (int)(r - M.ranges), w * r->grain, write ? "write" : "read", M.cur,
+                    what, other);
       if (M.races.size() < 20) M.races.insert(msg);
     };
     if (x.writer >= 0 && x.writer != M.cur && x.at > t.vc[x.writer]) race("write", x.writer);
     if (write) {
-      for (auto& r : x.reads)
-        if (r.first != M.cur && r.second > t.vc[r.first]) race("read", r.first);
+      if (x.read)
+        for (int k = 0; k < M.count; ++k)
+          if (k != M.cur && x.reads[k] > t.vc[k]) race("read", k);
       x.writer = M.cur;
       x.at = t.vc[M.cur];
-      x.reads.clear();
+      x.read = false;
     } else {
+      if (!x.read) x.reads = Clock();
+      x.read = true;
       x.reads[M.cur] = t.vc[M.cur];
     }
   }
 }
-
 LANES_RAW inline void access(const void* p, size_t bytes, bool write) {
   if (checking || !machine || machine->cur < 0) return;
   checking = true;
@@ -114,62 +139,57 @@ LANES_RAW inline void access(const void* p, size_t bytes, bool write) {
 
 LANES_RAW inline void yield() {
   const int c = m().cur;
-  swapcontext(&m().th[c].ctx, &m().main);
+  swapcontext(&m().threads[c].ctx, &m().main);
 }
 
 enum : int { ORDERED = 1, EXCHANGE = 2, BLOCK = 3 };
-// Meets the threads of mask in this warp (kind BLOCK: all that are not done) and
-// returns the values they brought, by lane.
-LANES_RAW inline std::vector<uint64_t> meet(int kind, unsigned mask, uint64_t value) {
-  Thread& t = me();
+// Meets the threads of mask in this warp (kind BLOCK: all that are not done).  An
+// exchange leaves the values that the lanes brought in got[32].
+LANES_RAW inline void meet(int kind, unsigned mask, uint64_t value, uint64_t* got = nullptr) {
+  Machine& M = m();
+  Thread* th = M.threads;
+  Thread& t = th[M.cur];
   t.waits = kind;
   t.mask = mask;
   t.value = value;
   while (t.waits) yield();
-  std::vector<uint64_t> got(32, 0);
-  const int w0 = m().cur & ~31;
-  for (int k = 0; k < 32 && w0 + k < (int)m().th.size(); ++k) got[k] = m().th[w0 + k].value;
-  if (kind == EXCHANGE) {  // everyone has read before anyone goes on
-    t.waits = kind;
-    while (t.waits) yield();
-  }
-  return got;
+  if (!got) return;
+  const int w0 = M.cur & ~31;
+  for (int k = 0; k < 32; ++k) got[k] = mask >> k & 1u ? th[w0 + k].value : 0;
+  t.waits = kind;  // everyone has read before anyone goes on
+  while (t.waits) yield();
 }
 
 // Lets those go on whose meeting is complete.
 LANES_RAW inline bool release() {
   Machine& M = m();
+  Thread* th = M.threads;
+  const int n = M.count;
   bool any = false;
-  const int n = (int)M.th.size();
   for (int k = 0; k < n; ++k) {
-    Thread& t = M.th[k];
+    Thread& t = th[k];
     if (t.done || !t.waits) continue;
-    std::vector<int> all;
+    const int kind = t.waits, from = kind == BLOCK ? 0 : k & ~31, to = kind == BLOCK ? n : from + 32;
+    auto in = [&](int j) LANES_RAW { return kind == BLOCK ? !th[j].done : (t.mask >> (j & 31) & 1u) != 0; };
     bool complete = true;
-    if (t.waits == BLOCK) {
-      for (int j = 0; j < n; ++j)
-        if (!M.th[j].done) {
-          all.push_back(j);
-          complete = complete && M.th[j].waits == BLOCK;
-        }
-    } else {
-      for (int j = 0; j < 32; ++j)
-        if (t.mask >> j & 1u) {
-          const int o = (k & ~31) + j;
-          all.push_back(o);
-          complete = complete && !M.th[o].done && M.th[o].waits == t.waits && M.th[o].mask == t.mask;
-        }
-    }
+    for (int j = from; j < to && complete; ++j)
+      if (in(j))
+        complete = !th[j].done && th[j].waits == kind && (kind == BLOCK || th[j].mask == t.mask);
     if (!complete) continue;
-    if (t.waits != EXCHANGE) {
-      Clock joint(n, 0);
-      for (int j : all) join(joint, M.th[j].vc);
-      for (int j : all) {
-        M.th[j].vc = joint;
-        ++M.th[j].vc[j];
-      }
+    if (kind != EXCHANGE) {
+      uint32_t* joint = M.joint;
+      for (int c = 0; c < n; ++c) joint[c] = 0;
+      for (int j = from; j < to; ++j)
+        if (in(j))
+          for (int c = 0; c < n; ++c) joint[c] = th[j].vc[c] > joint[c] ? th[j].vc[c] : joint[c];
+      for (int j = from; j < to; ++j)
+        if (in(j)) {
+          for (int c = 0; c < n; ++c) th[j].vc[c] = joint[c];
+          ++th[j].vc[j];
+        }
     }
-    for (int j : all) M.th[j].waits = 0;
+    for (int j = from; j < to; ++j)
+      if (in(j)) th[j].waits = 0;
     any = true;
   }
   return any;
@@ -185,18 +205,21 @@ LANES_RAW inline void entry() {
 // picks.  Returns the number of distinct races found (printed).
 LANES_RAW inline int run(int threads, unsigned seed, std::function<void()> body) {
   Machine& M = m();
-  M.th.clear();
-  M.th.resize(threads);
-  M.words.clear();
+  std::vector<Thread> store(threads);
+  M.threads = store.data();
+  M.count = threads;
+  for (Range& r : M.watched) {
+    r.words.assign(r.bytes / r.grain + 1, Word());
+    r.table = r.words.data();
+  }
+  M.ranges = M.watched.data();
+  M.range_count = (int)M.watched.size();
   M.races.clear();
   M.body = body;
   for (int k = 0; k < threads; ++k) {
-    Thread& t = M.th[k];
+    Thread& t = M.threads[k];
     t.tid = dim3(k, 0, 0);
-    t.vc.assign(threads, 0);
     t.vc[k] = 1;
-    t.released.assign(threads, 0);
-    t.pending.assign(threads, 0);
     t.stack.resize(256 << 10);
     getcontext(&t.ctx);
     t.ctx.uc_stack.ss_sp = t.stack.data();
@@ -204,7 +227,7 @@ LANES_RAW inline int run(int threads, unsigned seed, std::function<void()> body)
     t.ctx.uc_link = &M.main;
     makecontext(&t.ctx, entry, 0);
   }
-  for (auto& a : M.atomics) a.second.assign(threads, 0);
+  for (auto& a : M.atomics) a.second = Clock();
   uint64_t rng = 0x9e3779b97f4a7c15ull * (seed + 1);
   std::vector<int> order(threads);
   for (int k = 0; k < threads; ++k) order[k] = k;
@@ -215,7 +238,7 @@ LANES_RAW inline int run(int threads, unsigned seed, std::function<void()> body)
       std::swap(order[k], order[(rng >> 33) % (k + 1)]);
     }
     for (int k : order) {
-      Thread& t = M.th[k];
+      Thread& t = M.threads[k];
       left = left || !t.done;
       if (t.done || t.waits) continue;
       M.cur = k;
@@ -255,14 +278,15 @@ LANES_RAW inline void fence() {
 template <class T, class F>
 LANES_RAW inline T rmw(T* p, F f) {
   Clock& c = m().atomics[(uintptr_t)p];
-  if (c.empty()) c.assign(m().th.size(), 0);
   join(me().pending, c);
   join(c, me().released);
   const T old = *p;
   *p = f(old);
   return old;
 }
-LANES_RAW inline void watch(const void* p, size_t bytes) { m().watched[(uintptr_t)p] = bytes; }
+LANES_RAW inline void watch(const void* p, size_t bytes, size_t grain = 4) {
+  m().watched.push_back({(uintptr_t)p, bytes, grain, {}, nullptr});
+}
 LANES_RAW inline void atomic_word(const void* p) { m().atomics[(uintptr_t)p]; }
 
 inline float reciprocal(const char* text, float v) {
@@ -306,7 +330,7 @@ LANES_RAW void __tsan_vptr_read(void**) {}
 // ------------------------------------------------------------- device built-ins
 #define threadIdx (lanes::me().tid)
 static const dim3 blockIdx(0, 0, 0), gridDim(1, 1, 1);
-#define blockDim (dim3((unsigned)lanes::m().th.size(), 1, 1))
+#define blockDim (dim3((unsigned)lanes::m().count, 1, 1))
 
 LANES_RAW inline void __syncwarp(unsigned mask = 0xffffffffu) { lanes::meet(lanes::ORDERED, mask, 0); }
 LANES_RAW inline void __syncthreads() { lanes::meet(lanes::BLOCK, 0, 0); }
@@ -315,16 +339,21 @@ inline void __threadfence() { lanes::fence(); }
 inline void __threadfence_system() { lanes::fence(); }
 template <class T>
 LANES_RAW inline T __shfl_sync(unsigned mask, T v, int src, int = 32) {
-  return lanes::unpack<T>(lanes::meet(lanes::EXCHANGE, mask, lanes::pack(v))[src & 31]);
+  uint64_t got[32];
+  lanes::meet(lanes::EXCHANGE, mask, lanes::pack(v), got);
+  return lanes::unpack<T>(got[src & 31]);
 }
 template <class T>
 LANES_RAW inline T __shfl_xor_sync(unsigned mask, T v, int o, int = 32) {
   const int lane = lanes::m().cur & 31;
-  return lanes::unpack<T>(lanes::meet(lanes::EXCHANGE, mask, lanes::pack(v))[(lane ^ o) & 31]);
+  uint64_t got[32];
+  lanes::meet(lanes::EXCHANGE, mask, lanes::pack(v), got);
+  return lanes::unpack<T>(got[(lane ^ o) & 31]);
 }
 template <class F>
 LANES_RAW inline unsigned lanes_reduce(unsigned mask, unsigned v, F f) {
-  const auto got = lanes::meet(lanes::EXCHANGE, mask, v);
+  uint64_t got[32];
+  lanes::meet(lanes::EXCHANGE, mask, v, got);
   bool first = true;
   unsigned r = 0;
   for (int k = 0; k < 32; ++k)
@@ -342,7 +371,8 @@ inline unsigned __reduce_or_sync(unsigned mask, unsigned v) {
 }
 inline int __any_sync(unsigned mask, int p) { return __reduce_or_sync(mask, p != 0) != 0; }
 LANES_RAW inline unsigned __ballot_sync(unsigned mask, int p) {
-  const auto got = lanes::meet(lanes::EXCHANGE, mask, p != 0);
+  uint64_t got[32];
+  lanes::meet(lanes::EXCHANGE, mask, p != 0, got);
   unsigned r = 0;
   for (int k = 0; k < 32; ++k)
     if (mask >> k & 1u) r |= (unsigned)(got[k] & 1u) << k;

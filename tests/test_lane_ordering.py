@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 CUDA = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
 
 
-@pytest.mark.parametrize("program", ["solve_share"])
+@pytest.mark.parametrize("program", ["solve_share", "hand_over"])
 def test_accesses_are_ordered(program, tmp_path):
     gxx = shutil.which("g++")
     if gxx is None or not os.path.exists(os.path.join(CUDA, "cuda_runtime.h")):
@@ -21,7 +21,7 @@ def test_accesses_are_ordered(program, tmp_path):
     exe = str(tmp_path / program)
     src = os.path.join(HERE, "lanes", program + ".cpp")
     # compiled with the sanitizer's calls, linked without its library: lanes.h has them
-    subprocess.check_call([gxx, "-std=c++17", "-O1", "-w", "-fsanitize=thread",
+    subprocess.check_call([gxx, "-std=c++17", "-O2", "-w", "-fsanitize=thread",
                            "-ffp-contract=off", "-I" + CUDA, "-I" + os.path.join(ROOT, "include"),
                            "-I" + os.path.join(ROOT, "paper_2112_03444_gb300", "csrc"),
                            "-c", src, "-o", exe + ".o"])
