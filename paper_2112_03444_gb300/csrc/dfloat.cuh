@@ -367,7 +367,8 @@ __device__ __forceinline__ bool gj_solve_df(const Group& g, cx<df>* A, cx<df>* p
       cx<df> a[UNROLL];
 #pragma unroll
       for (int u = 0; u < UNROLL; ++u) {
-        const int ju = min(j + u * PARTS, W - 1);
+        // (behind the last column: this lane's own j, as another lane may be storing W - 1)
+        const int ju = j + u * PARTS < W ? j + u * PARTS : j;
         const cx<df> p = pv[ju];
         a[u] = dot2p(A[ju * LR + r], lr, p, li, im_re(p));
       }

@@ -244,6 +244,7 @@ struct TermBlock {
     eval_share(t, want);
     H = Hs()[i];
     Ht = A()[LR * N + (i & (LR - 1))];
+    __syncwarp();  // the first replica's lanes put the right-hand side in its place
   }
 
   template <class R>

@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 CUDA = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
 
 
-@pytest.mark.parametrize("program", ["solve_share", "hand_over"])
+@pytest.mark.parametrize("program", ["solve_share", "hand_over", "trackers"])
 def test_accesses_are_ordered(program, tmp_path):
     gxx = shutil.which("g++")
     if gxx is None or not os.path.exists(os.path.join(CUDA, "cuda_runtime.h")):
