@@ -230,6 +230,7 @@ struct TermEval {
   template <bool SCALE, int EP = 1>
   __device__ __forceinline__ void residual64(const cx<double>*, int i, double t, double,
                                              cx<double>& H, double& sc) const {
+    __syncwarp(g.mask);  // the evaluation has read p(t)
     put_params<double>(t, g.mask);
     const int rr = i & (ROWL - 1), part = i / ROWL;
     const int ii = rr < N ? rr : 0;

@@ -623,7 +623,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
           const int code = hand_code(e);
           inst_cur = item / c.paths;
           hom = prob.hom(inst_cur);
-          hom.init(g);
+          hom.init(g);  // (behind the __syncwarp above: the last path's values are read)
           const float2* slot = reinterpret_cast<const float2*>(c.x_out + item * (2 * N));
           const float2 v = act ? __ldcg(slot + g.gl) : make_float2(0.f, 0.f);
           const float2 tt = __ldcg(slot + N);
@@ -683,6 +683,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         const int64_t k_in = item - inst * c.paths;
         const int64_t path = c.path_ids ? c.path_ids[item] : c.path_map ? c.path_map[k_in] : k_in;
         hom = prob.hom(inst);
+        __syncwarp(g.mask);  // the last path's values are read
         hom.init(g);  // per-path constants of the evaluator (shared memory)
         // a path handed over by the FP32 tier resumes from its last accepted point
         const double t0 = (!MIXED && c.t_io) ? c.t_io[item] : 0.0;
@@ -1062,6 +1063,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
             hom.template residual64<true>(sm.vd, g.gl, 1.0, 0.0, H64, sc);
             r = (double)cabs2(cvt<float>(H64));
           }
+          __syncwarp(g.mask);  // the point copy is read
           const double bei = act ? (sc > 0.0 ? r / sc : r) : 0.0;
           be = gmaxf(g, (float)bei);
           if (!((double)be <= s.finite_tol)) {

@@ -4,6 +4,7 @@
 
 #include "dense_kernel.cuh"
 #include "term_block.cuh"
+#include "term_param.cuh"
 
 static hc::DevSettings settings() {
   hc::DevSettings s;
@@ -158,6 +159,23 @@ int family_df(unsigned seed, int items) {
   });
 }
 
+template <int N, int L, bool MIXED>
+int family_rows(unsigned seed, int items) {
+  constexpr int LS = N <= 4 ? 4 : N <= 8 ? 8 : N <= 16 ? 16 : 32;
+  const int threads = 64, acc = hc::term_acc_bytes<N, MIXED, L>();
+  const int eg = hc::endgame_smem_bytes(L, MIXED);
+  const size_t smem = hc::block_smem_bytes(L, 4, acc, threads, eg);
+  return family<N>(seed, LS, 1, items, smem, hc::group_smem_bytes(L, 4, acc, eg) - 16,
+                   [&](hc::TermArgs& a, unsigned char* mem) {
+    return lanes::run(threads, seed, [&] {
+      const hc::Group g = hc::make_group<L, hc::groups_meet(L, false, MIXED)>();
+      const hc::GroupMem sm = hc::make_group_mem<L>(mem, a.extra, acc, eg);
+      hc::TermProblem<N, L, MIXED> prob{&a, g, sm};
+      hc::run_tracker<N, L, MIXED, hc::TermProblem<N, L, MIXED>, double>(prob, a.c, g, sm);
+    });
+  });
+}
+
 // Dense kernels on random tables: most steps are rejected, which reaches every phase.
 template <int N, int DEG, int PREC, int L>
 int dense(unsigned seed, int items) {
@@ -208,6 +226,11 @@ int main() {
     RUN(family_df<3, 1>(seed, 3))
     RUN(family_df<6, 2>(seed, 2))
     RUN(family_df<9, 4>(seed, 2))
+    RUN((family_rows<3, 4, true>(seed, 20)))
+    RUN((family_rows<6, 8, false>(seed, 6)))
+    RUN((family_rows<9, 16, true>(seed, 6)))
+    RUN((family_rows<9, 16, false>(seed, 3)))
+    RUN((family_rows<5, 32, true>(seed, 3)))
     RUN((dense<3, 2, HC_PREC_MIXED, 4>(seed, 20)))
     RUN((dense<5, 3, HC_PREC_MIXED, 8>(seed, 9)))
     RUN((dense<9, 2, HC_PREC_FP64, 16>(seed, 4)))
