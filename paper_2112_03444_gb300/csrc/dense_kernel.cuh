@@ -55,26 +55,26 @@ constexpr int kTrackMinBlocks = 4;
 // 13.3 -> 14.5 / 21.0 ms, precision DF on it 433 -> 419 / 448 ms.  Two or four
 // warps per path (columns over the warps) lose as well: re-tracking 13.2 / 11.6
 // ms, precision DF 782 / 1070 ms.
-template <int N, int DEG, int PREC, int L, bool RING = false>
+template <int N, int DEG, int PREC, int L, int FORM = F_BATCH>
 __global__ void __launch_bounds__(kBlock, PREC == HC_PREC_DF ? 1 : kTrackMinBlocks)
     dense_td_kernel(const DenseArgs a) {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
   constexpr bool XDF = PREC == HC_PREC_DF;
   using RE = typename std::conditional<XDF, df, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L, groups_meet(L, RING, MIXED)>();
+  const Group g = make_group<L, groups_meet(L, FORM == F_RING, MIXED)>();
   const GroupMem sm = make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(),
                                         endgame_smem_bytes(L, MIXED), XDF ? 1 : 0);
   DenseProblem<N, DEG, L> prob{&a, sm, g.meet};
-  run_tracker<N, L, MIXED, DenseProblem<N, DEG, L>, RE, RING>(prob, a.c, g, sm);
+  run_tracker<N, L, MIXED, DenseProblem<N, DEG, L>, RE, FORM>(prob, a.c, g, sm);
 }
 
 // lanes = 0: the default lanes_for(N); otherwise that group width.  RING:
 // the resident-launch variant (hc_stream).
-template <int DEG, int PREC, int N, int LANES = 0, bool RING = false>
+template <int DEG, int PREC, int N, int LANES = 0, int FORM = F_BATCH>
 KernelRef dense_ref() {
   constexpr int L = LANES ? LANES : ((N <= 4) ? 4 : (N <= 8) ? 8 : (N <= 16) ? 16 : 32);
-  return KernelRef{reinterpret_cast<const void*>(&dense_td_kernel<N, DEG, PREC, L, RING>), L,
+  return KernelRef{reinterpret_cast<const void*>(&dense_td_kernel<N, DEG, PREC, L, FORM>), L,
                    DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(),
                    endgame_smem_bytes(L, PREC == HC_PREC_MIXED),
                    PREC == HC_PREC_DF ? 1 : 0};

@@ -1778,7 +1778,8 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
       ta.dcf = B.dcf;
       ta.dcdf = B.dcdf;
     }
-    const hc::KernelRef k = hc::term_kernel(n, p->s.precision, mixed ? p->s.lanes : 0);
+    hc::KernelRef k = hc::term_kernel(n, p->s.precision, mixed ? p->s.lanes : 0);
+    if (mixed && B.step_budget > 0 && k.lanes < 32) k = hc::budget_kernel(true, 0, n);
     auto smem_of = [&](const hc::KernelRef& kr, int threads = hc::kBlock) {
       return (size_t)hc::block_smem_bytes(kr.lanes, p->extra, kr.acc_bytes, threads, kr.eg_bytes,
                                           kr.vx, kr.warps);
@@ -1834,7 +1835,9 @@ hc_status enqueue_compute(hc_problem* p, int64_t n_inst, const Bufs& B, cudaStre
     a.gamma = cx<double>{p->gamma[0], p->gamma[1]};
     a.gamma32 = cx<float>{(float)p->gamma[0], (float)p->gamma[1]};
     a.gammadf = hc::split_cdf_host(p->gamma[0], p->gamma[1]);
-    const hc::KernelRef k = hc::dense_kernel(p->deg, n, p->s.precision, mixed ? p->s.lanes : 0);
+    hc::KernelRef k = hc::dense_kernel(p->deg, n, p->s.precision, mixed ? p->s.lanes : 0);
+    if (mixed && B.step_budget > 0 && k.fn && k.lanes < 32)
+      k = hc::budget_kernel(false, p->deg, n);
     if (!k.fn) {
       set_err("no kernel for this problem shape");
       return HC_ERR_UNSUPPORTED;

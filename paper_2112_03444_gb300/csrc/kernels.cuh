@@ -234,6 +234,9 @@ inline int lanes_for(int n) { return n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32
 
 // prec: HC_PREC_FP64, HC_PREC_MIXED or HC_PREC_DF.  lanes = 0: default
 // group width; 32: one path per warp (mixed kernels, n <= 16)
+// The form of a tracking kernel: a batch's, the resident launch of a stream, or a
+// batch's with a step budget (mixed kernels with several paths per warp).
+enum : int { F_BATCH = 0, F_RING = 1, F_BUDGET = 2 };
 KernelRef dense_kernel(int deg, int n, int prec, int lanes);  // fn == nullptr if absent
 KernelRef term_kernel(int n, int prec, int lanes);            // fn == nullptr if absent
 // Kernel of the re-tracking tiers (few paths): one path per warp with split
@@ -250,6 +253,8 @@ inline int last_tier_precision(const hc_settings& s) {
 // Resident-launch (hc_stream) variant of the mixed tracking kernel for a
 // problem: term tables or dense of degree deg; fn == nullptr if absent.
 KernelRef ring_kernel(bool terms, int deg, int n);
+// The kernels of batches with a step budget; fn == nullptr if absent.
+KernelRef budget_kernel(bool terms, int deg, int n);
 
 // Evaluation kernels of hc_evaluate (prec: HC_PREC_FP64, HC_PREC_MIXED =
 // FP32 evaluation, HC_PREC_DF); fn == nullptr if absent.

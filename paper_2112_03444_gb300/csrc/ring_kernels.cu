@@ -12,7 +12,7 @@ KernelRef pick_dense_ring(int n) {
   if constexpr (N == 0)
     return KernelRef{nullptr, 0};
   else
-    return n == N ? dense_ref<DEG, HC_PREC_MIXED, N, 0, true>() : pick_dense_ring<DEG, N - 1>(n);
+    return n == N ? dense_ref<DEG, HC_PREC_MIXED, N, 0, F_RING>() : pick_dense_ring<DEG, N - 1>(n);
 }
 
 template <int N>
@@ -20,7 +20,7 @@ KernelRef pick_term_ring(int n) {
   if constexpr (N == 0)
     return KernelRef{nullptr, 0};
   else
-    return n == N ? term_ref<HC_PREC_MIXED, N, 0, true>() : pick_term_ring<N - 1>(n);
+    return n == N ? term_ref<HC_PREC_MIXED, N, 0, F_RING>() : pick_term_ring<N - 1>(n);
 }
 
 KernelRef ring_kernel(bool terms, int deg, int n) {

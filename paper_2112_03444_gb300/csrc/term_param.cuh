@@ -317,22 +317,22 @@ __host__ __device__ constexpr int term_acc_bytes() {
 }
 
 // PREC: HC_PREC_MIXED or HC_PREC_FP64 (double-float: term_block.cuh)
-template <int N, int PREC, int L, bool RING = false>
+template <int N, int PREC, int L, int FORM = F_BATCH>
 __global__ void __launch_bounds__(kBlock) term_param_kernel(const __grid_constant__ TermArgs a) {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L, groups_meet(L, RING, MIXED)>();
+  const Group g = make_group<L, groups_meet(L, FORM == F_RING, MIXED)>();
   const GroupMem sm = make_group_mem<L>(smem, a.extra, term_acc_bytes<N, MIXED, L>(),
                                         endgame_smem_bytes(L, MIXED));
   TermProblem<N, L, MIXED> prob{&a, g, sm};
-  run_tracker<N, L, MIXED, TermProblem<N, L, MIXED>, double, RING>(prob, a.c, g, sm);
+  run_tracker<N, L, MIXED, TermProblem<N, L, MIXED>, double, FORM>(prob, a.c, g, sm);
 }
 
-template <int PREC, int N, int LANES = 0, bool RING = false>
+template <int PREC, int N, int LANES = 0, int FORM = F_BATCH>
 KernelRef term_ref() {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
   constexpr int L = LANES ? LANES : ((N <= 4) ? 4 : (N <= 8) ? 8 : (N <= 16) ? 16 : 32);
-  return KernelRef{reinterpret_cast<const void*>(&term_param_kernel<N, PREC, L, RING>), L, 0,
+  return KernelRef{reinterpret_cast<const void*>(&term_param_kernel<N, PREC, L, FORM>), L, 0,
                    term_acc_bytes<N, MIXED, L>(), endgame_smem_bytes(L, MIXED), 0};
 }
 

@@ -244,6 +244,8 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
                                           const GroupMem& sm) {
   static_assert(PHASE == P_WHOLE || (MIXED && !RING), "phases: mixed kernels of a batch");
   constexpr bool LOW = PHASE == P_LOW;
+  // the launches of a batch with a step budget have one loop (run_tracker)
+  constexpr bool BUDGET = PHASE == P_WHOLE;
   using R = typename std::conditional<MIXED, float, RE>::type;
   using HOM = decltype(prob.hom(0));
   // double-float kernels: their Newton corrector takes its residual in FP64
@@ -300,7 +302,6 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
   double t = 0.0, dt = 0.0, h = 0.0, t1 = 0.0;
   float tf = 0.f, dtf = 0.f, hf = 0.f, t1f = 0.f;
   int consec = 0, nacc = 0, nrej = 0, nnewt = 0, status = 0;
-  int counted = 0;  // steps of the path already added to *step_total (P_HIGH)
   int mode = M_FETCH, stage = 0, it = 0;
   cx<R> kprev = czero<R>(), ksum = czero<R>();
   cx<float> xpf = czero<float>();   // corrector iterate (FP32 state)
@@ -342,7 +343,6 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
       c.steps_out[item * 3 + 1] = nrej;
       c.steps_out[item * 3 + 2] = nnewt;
       if (code == H_DONE) c.status_out[item] = (uint8_t)status;
-      if (c.step_budget) atomicAdd(c.step_total, (unsigned long long)(nacc + nrej));
     }
     __threadfence_block();
     __syncwarp(g.mask);
@@ -509,8 +509,8 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
       if (g.gl == 0) {
         c.status_out[item] = (uint8_t)status;
         if (c.be_out) c.be_out[item] = (double)be;
-        if (c.step_budget)
-          atomicAdd(c.step_total, (unsigned long long)(nacc + nrej - counted));
+        if (BUDGET && c.step_budget)
+          atomicAdd(c.step_total, (unsigned long long)(nacc + nrej));
         if (MIXED) {
           c.steps_out[item * 3 + 0] = nacc;
           c.steps_out[item * 3 + 1] = nrej;
@@ -634,7 +634,6 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
           nacc = __ldcg(c.steps_out + item * 3 + 0);
           nrej = __ldcg(c.steps_out + item * 3 + 1);
           nnewt = __ldcg(c.steps_out + item * 3 + 2);
-          counted = nacc + nrej;
           status = code == H_DONE ? (int)__ldcg(c.status_out + item) : 0;
           res64 = false;
           be = 0.f;
@@ -651,7 +650,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
     }
     if (mode == M_FETCH) {
       bool stop = false;  // no further path for this group
-      if (c.step_budget && !c.items) {
+      if (BUDGET && c.step_budget && !c.items) {
         // the budget stops new paths of the launch; started ones finish
         unsigned long long spent = 0;
         if (g.gl == 0) spent = *reinterpret_cast<volatile unsigned long long*>(c.step_total);
@@ -703,7 +702,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         dt = s.dt_init;
         tf = (float)t;
         dtf = (float)s.dt_init;
-        consec = nacc = nrej = nnewt = status = counted = 0;
+        consec = nacc = nrej = nnewt = status = 0;
         res64 = false;
         be = 0.f;
         // endgame: the first sample time after the start point
@@ -1119,15 +1118,23 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
 // its items are few and long, and the second loop would wait for the warp's own
 // paths (trifocal, 4 scenes: 184 -> 206 with two loops).
 //
+// A step budget stops new paths once the finished ones took that many steps, which
+// the first loop cannot know: the launches of such a batch take kernels with one loop
+// (F_BUDGET), where no more paths are begun and unfinished than there are groups.
+// They are kernels of their own: a branch to one loop cost the two others registers
+// (n = 14 term tables 128 -> 159), and both loops in turn, one path per group in the
+// first, cost one quadratic n = 6 system and P3P 2 %.
+//
 // The second loop waits for nothing: a path goes onto its block's hand-over
 // list from its warp's first loop, so the warp that handed over last still has
 // its second loop ahead, where it takes every path the others left.  (One list
 // for the whole grid loses more to the contention on its head than its balance
 // gives: cubic n = 8, 40 -> 190 ms with a compare-and-swap per path.)
-template <int N, int L, bool MIXED, class PROB, class RE = double, bool RING = false>
+template <int N, int L, bool MIXED, class PROB, class RE = double, int FORM = F_BATCH>
 __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon& c,
                                             const Group& g, const GroupMem& sm) {
-  if constexpr (MIXED && groups_meet(L, RING, MIXED)) {
+  constexpr bool RING = FORM == F_RING;
+  if constexpr (FORM == F_BATCH && MIXED && groups_meet(L, RING, MIXED)) {
     if (!c.start_hi) {
       if (threadIdx.x == 0) *sm.hand = 0;
       __syncthreads();

@@ -1,6 +1,7 @@
 // The two loops of the mixed tracking kernels (run_tracker): what the first loop
 // hands over is ordered before the second loop's reads, and every path is finished
-// once.  The problem: x_i' = 1 from 1 + i at t = 0, an identity Jacobian.
+// once -- or, under a step budget, as many as it allows.  The problem: x_i' = 1 from
+// 1 + i at t = 0, an identity Jacobian.
 #include "lanes.h"
 
 #include "tracker.cuh"
@@ -85,8 +86,20 @@ int check(unsigned seed, int warps, int items, int max_steps_fp32, unsigned long
   int bad = lanes::run(32 * warps, seed, [&] {
     const hc::Group g = hc::make_group<L, true>();
     const hc::GroupMem sm = hc::make_group_mem<L>(mem, 0);
-    hc::run_tracker<N, L, true, StraightProblem<N, L>>(StraightProblem<N, L>{sm}, c, g, sm);
+    const StraightProblem<N, L> prob{sm};
+    if (budget)
+      hc::run_tracker<N, L, true, StraightProblem<N, L>, double, hc::F_BUDGET>(prob, c, g, sm);
+    else
+      hc::run_tracker<N, L, true, StraightProblem<N, L>>(prob, c, g, sm);
   });
+  int begun = 0;
+  for (int k = 0; k < items; ++k) begun += steps[3 * k] != 0;
+  const int groups = 32 / L * warps;
+  // a path takes 10 steps at least: three finished ones exceed 26
+  if (budget == 26 && begun > groups + 2) {
+    std::printf("%d paths begun by %d groups under a budget of two paths\n", begun, groups);
+    return bad + 1;
+  }
   for (int k = 0; k < items; ++k)
     if ((status[k] & 0x7f) != 1 || std::fabs(x[2 * N * k] - 2.0) > 1e-10 || steps[3 * k] < 10) {
       if (budget && !status[k]) continue;
@@ -100,6 +113,7 @@ int main() {
   int bad = 0;
   for (unsigned seed = 0; seed < 3; ++seed)
     bad += check<2, 4>(seed, 1, 20, 1000, 0) + check<3, 8>(seed, 2, 30, 1000, 0) +
-           check<3, 16>(seed, 3, 17, 3, 0) + check<2, 8>(seed, 2, 9, 1, 0);
+           check<3, 16>(seed, 3, 17, 3, 0) + check<2, 8>(seed, 2, 9, 1, 0) +
+           check<2, 8>(seed, 2, 60, 1, 26) + check<2, 8>(seed, 2, 20, 5, 1ull << 40);
   return bad != 0;
 }
