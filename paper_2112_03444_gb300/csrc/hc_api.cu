@@ -2032,8 +2032,13 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
   bt->admission = adm;
   const int64_t items = bt->items;
   cudaStream_t st = bt->stream;
+  cudaStream_t hs = nullptr, hs2 = nullptr;  // of the re-tracking, once taken
   auto fail = [&](hc_status s) {
-    cudaDeviceSynchronize();  // the re-tracking streams may hold launches of the batch
+    // what the batch may have in flight, and nothing else: the device may hold
+    // launches that end only when their streams do (hc_stream)
+    cudaStreamSynchronize(st);
+    if (hs) cudaStreamSynchronize(hs);
+    if (hs2) cudaStreamSynchronize(hs2);
     release_batch(bt);
     if (cur != p->device) cudaSetDevice(cur);
     return s;
@@ -2128,8 +2133,9 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
   bt->d_ctl = B.d_ctl;
   // ---- the computation
   const EnqEvents ev{bt->evk0, bt->evk1, bt->evk2, nullptr, nullptr, bt->evf, bt->evj, false};
-  const cudaStream_t hs = retrack_stream(p->device);
-  HC_TRY(enqueue_compute(p, bt->n_inst, B, st, hs, retrack_stream(p->device), ev));
+  hs = retrack_stream(p->device);
+  hs2 = retrack_stream(p->device);
+  HC_TRY(enqueue_compute(p, bt->n_inst, B, st, hs, hs2, ev));
   for (size_t i = 0; i < bt->copies.size(); ++i) {
     void* dst = bt->copies[i].pinned ? bt->copies[i].pinned : bt->copies[i].dst;
     HC_TRYCUDA(cudaMemcpyAsync(dst, d2h[i], bt->copies[i].bytes, cudaMemcpyDeviceToHost, st));
