@@ -2041,6 +2041,7 @@ hc_status hc_track_batch(hc_problem* p, const hc_batch_desc* b, hc_batch** out) 
     if (hs2) cudaStreamSynchronize(hs2);
     release_batch(bt);
     if (cur != p->device) cudaSetDevice(cur);
+    cudaGetLastError();  // reported by s: the caller's next calls find none
     return s;
   };
   std::function<hc_status(size_t, void**)> dalloc = [&](size_t bytes, void** q) -> hc_status {
@@ -2209,6 +2210,7 @@ hc_status hc_plan_create(hc_problem* p, int32_t n_instances, hc_plan** out) {
   auto fail = [&](hc_status s) {
     free_plan(pl);
     if (cur != p->device) cudaSetDevice(cur);
+    cudaGetLastError();  // reported by s: the caller's next calls find none
     return s;
   };
   auto dalloc = [&](size_t bytes, void** q) -> hc_status {
@@ -2320,6 +2322,7 @@ hc_status hc_plan_run(hc_plan* pl, const hc_batch_desc* b, hc_batch** out) {
     cudaStreamSynchronize(st);
     release_batch(bt);
     if (cur != p->device) cudaSetDevice(cur);
+    cudaGetLastError();  // reported by s: the caller's next calls find none
     return s;
   };
 #define HC_TRYCUDA(call)                                           \
@@ -2653,6 +2656,7 @@ extern "C" hc_status hc_evaluate(const hc_problem* p, int32_t precision, int32_t
       return HC_ERR_INVALID;
     }
   if (n_points == 0) return HC_OK;
+  cudaGetLastError();  // launch errors checked below are this call's own
   const hc::KernelRef k = p->terms ? hc::term_eval_kernel(p->n, precision)
                                    : hc::dense_eval_kernel(p->deg, p->n, precision);
   if (!k.fn) {
@@ -3226,6 +3230,7 @@ extern "C" hc_status hc_stream_submit(hc_stream* s, const double* inputs, int64_
     set_err("hc_stream_submit: invalid arguments");
     return HC_ERR_INVALID;
   }
+  cudaGetLastError();  // launch errors checked below are this call's own
   const hc_problem* p = s->p;
   const int64_t k = s->next_ticket;
   const int slot = (int)(k % s->S);

@@ -272,6 +272,7 @@ extern "C" hc_status hc_track_dense_noalloc(int32_t n, int32_t degree, const dou
       static_cast<unsigned char*>(base) + kNoAllocScratchBytes);
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  cudaGetLastError();  // launch errors checked below are this call's own
 #define NA_CUDA(call)                                                                   \
   do {                                                                                  \
     if ((call) != cudaSuccess) {                                                        \
