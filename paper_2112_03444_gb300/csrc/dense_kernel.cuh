@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kBlock, PREC == HC_PREC_DF ? 1 : kTrackMinBloc
   constexpr bool XDF = PREC == HC_PREC_DF;
   using RE = typename std::conditional<XDF, df, double>::type;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L, groups_meet(L, FORM == F_RING, MIXED)>();
+  const Group g = make_group<L, groups_meet(L, MIXED)>();
   const GroupMem sm = make_group_mem<L>(smem, DenseShape<N, DEG>::EXTRA, dense_acc_bytes<N, PREC>(),
                                         endgame_smem_bytes(L, MIXED), XDF ? 1 : 0);
   DenseProblem<N, DEG, L> prob{&a, sm, g.meet};

@@ -130,11 +130,7 @@ struct DenseTD {
   // tracker has every lane of the warp compute a share of it: the outer
   // index j is split over WP = 32 / L parts (zigzag, as for split rows), the
   // parts are added by a butterfly over the warp, and the group then holds
-  // the rows' residuals (the *_coop functions below).  Where a group must
-  // compute a residual alone (the resident-launch kernels, whose groups wait
-  // for work independently), it forms the same WP partial sums one after the
-  // other and adds them in the butterfly's order (the *_seq functions), so
-  // that both forms give the same bits.
+  // the rows' residuals (the *_coop functions below).
   static constexpr bool kCoop = (PARTS == 1 && L_GROUP < 32);
   static constexpr int WP = 32 / L;
 
@@ -372,17 +368,10 @@ struct DenseTD {
   // ratio test) is returned in sc.  Runtime loops: this code runs a few
   // times per path and must not crowd the tracking loop out of the
   // instruction cache.  Split over PARTS lanes like eval (outer index j).
-  // EP > 1 (groups narrower than a warp): the WP-part order of the
-  // cooperative form, computed by the group alone.
-  template <bool SCALE_T, int EP = 1>
+  template <bool SCALE_T>
   __device__ __forceinline__ void residual64(const cx<double>* xs, int i, double t, double omt,
                                              cx<double>& H, double& sc) const {
-    if constexpr (EP > 1) {
-      static_assert(EP == WP && kCoop, "sequential parts: groups narrower than a warp");
-      residual64_seq(xs, i, t, omt, SCALE_T, H, sc);
-    } else {
-      residual64_impl(xs, i, t, omt, SCALE_T, H, sc);
-    }
+    residual64_impl(xs, i, t, omt, SCALE_T, H, sc);
   }
 
   // partial sums of row r over the outer indices j of part `part` of a
@@ -469,25 +458,6 @@ struct DenseTD {
     residual64_finish(xs, r, t, omt, scale, F, Ssum, H, sc);
   }
 
-  // the WP parts one after the other, added in the butterfly's order
-  __device__ __forceinline__ void residual64_seq(const cx<double>* xs, int i, double t, double omt,
-                                                 bool scale, cx<double>& H, double& sc) const {
-    const int r = i & (L - 1);
-    cx<double> F[WP];
-    float S[WP];
-#pragma unroll
-    for (int p = 0; p < WP; ++p) residual64_part<WP>(xs, r, p, scale, F[p], S[p]);
-#pragma unroll
-    for (int w = 1; w < WP; w <<= 1) {
-#pragma unroll
-      for (int p = 0; p < WP; p += 2 * w) {
-        F[p] = F[p] + F[p + w];
-        S[p] = S[p] + S[p + w];
-      }
-    }
-    residual64_finish(xs, r, t, omt, scale, F[0], S[0], H, sc);
-  }
-
   // Cooperative form: called by every lane of the warp (wl = lane index)
   // for the group whose point xs is; lane wl computes part wl / L of row
   // wl mod L, and after the butterfly every lane holds its row's residual.
@@ -515,15 +485,10 @@ struct DenseTD {
   // FP32: its error is a small multiple of 2^-48 times the size of the terms
   // (the backward-error scale sc, formed as in residual64), far below the
   // tolerances the FP64 residual serves, and only the FP32 solve consumes it.
-  template <bool SCALE_T, int EP = 1>
+  template <bool SCALE_T>
   __device__ __forceinline__ void residual_df(const cdf* xs, int i, double t, cx<float>& H,
                                               float& sc) const {
-    if constexpr (EP > 1) {
-      static_assert(EP == WP && kCoop, "sequential parts: groups narrower than a warp");
-      residual_df_seq(xs, i, t, SCALE_T, H, sc);
-    } else {
-      residual_df_impl(xs, i, t, SCALE_T, H, sc);
-    }
+    residual_df_impl(xs, i, t, SCALE_T, H, sc);
   }
 
   __device__ static cdf part_sum_cdf(cdf v) {
@@ -623,25 +588,6 @@ struct DenseTD {
       }
     }
     residual_df_finish(xs, r, t, scale, F, Ssum, H, sc);
-  }
-
-  // the WP parts one after the other, added in the butterfly's order
-  __device__ __forceinline__ void residual_df_seq(const cdf* xs, int i, double t, bool scale,
-                                                  cx<float>& H, float& sc) const {
-    const int r = i & (L - 1);
-    cdf F[WP];
-    float S[WP];
-#pragma unroll
-    for (int p = 0; p < WP; ++p) residual_df_part<WP>(xs, r, p, scale, F[p], S[p]);
-#pragma unroll
-    for (int w = 1; w < WP; w <<= 1) {
-#pragma unroll
-      for (int p = 0; p < WP; p += 2 * w) {
-        F[p] = cdf_add(F[p], F[p + w]);
-        S[p] = S[p] + S[p + w];
-      }
-    }
-    residual_df_finish(xs, r, t, scale, F[0], S[0], H, sc);
   }
 
   // Cooperative form (as residual64_coop)

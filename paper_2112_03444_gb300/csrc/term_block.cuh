@@ -304,7 +304,7 @@ struct TermBlock {
     H = h;
     sc = s_abs;
   }
-  template <bool SCALE, int EP = 1>
+  template <bool SCALE>
   __device__ __forceinline__ void residual64(const cx<double>*, int, double t, double,
                                              cx<double>& H, double& sc) const {
     float s_abs;

@@ -227,7 +227,7 @@ struct TermEval {
     }
   }
 
-  template <bool SCALE, int EP = 1>
+  template <bool SCALE>
   __device__ __forceinline__ void residual64(const cx<double>*, int i, double t, double,
                                              cx<double>& H, double& sc) const {
     __syncwarp(g.mask);  // the evaluation has read p(t)
@@ -263,7 +263,7 @@ struct TermEval {
   // factors and coefficient (table sdf) as in residual64.  H is returned
   // rounded to FP32 (its error is a small multiple of 2^-48 times the
   // backward-error scale sc).
-  template <bool SCALE, int EP = 1>
+  template <bool SCALE>
   __device__ __forceinline__ void residual_df(const cdf*, int i, double t, cx<float>& H,
                                               float& sc) const {
     const int P = a->P, LS = a->ls;
@@ -321,7 +321,7 @@ template <int N, int PREC, int L, int FORM = F_BATCH>
 __global__ void __launch_bounds__(kBlock) term_param_kernel(const __grid_constant__ TermArgs a) {
   constexpr bool MIXED = PREC == HC_PREC_MIXED;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Group g = make_group<L, groups_meet(L, FORM == F_RING, MIXED)>();
+  const Group g = make_group<L, groups_meet(L, MIXED)>();
   const GroupMem sm = make_group_mem<L>(smem, a.extra, term_acc_bytes<N, MIXED, L>(),
                                         endgame_smem_bytes(L, MIXED));
   TermProblem<N, L, MIXED> prob{&a, g, sm};

@@ -80,14 +80,16 @@ namespace hc {
 enum : int { M_RK = 0, M_NEWTON = 1, M_REFINE = 2, M_COND = 3, M_DONE = 4, M_FETCH = 5, M_IDLE = 6 };
 
 // Kernels whose warps hold several groups and keep them in step (see
-// make_group); the groups of a resident launch wait for work on their own.
+// make_group).
 // The all-FP64 kernels meet with two groups per warp only: an FP64 instruction
 // holds its pipe as long for one group as for all, and with four or eight groups
 // waiting for the slowest costs more than their separate instructions (ms, apart /
 // meeting: quadratic n = 6, 64 systems, 14.4 / 14.8; cubic n = 5, 24 systems, 29.3 /
-// 30.6; quadratic n = 12, 16 systems, two groups, 802 / 797).
-__host__ __device__ constexpr bool groups_meet(int L, bool ring, bool mixed) {
-  return !ring && L < 32 && (mixed || L == 16);
+// 30.6; quadratic n = 12, 16 systems, two groups, 811 / 807; with two groups the two
+// are within 1 % at 1 to 16 quadratic n = 9..11 systems and for 4-view triangulation
+// and relative pose).
+__host__ __device__ constexpr bool groups_meet(int L, bool mixed) {
+  return L < 32 && (mixed || L == 16);
 }
 
 // Phases of the mixed kernels: the whole path in one loop (resident launches),
@@ -197,6 +199,11 @@ __device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ unsigned int ld_relaxed_gpu(const unsigned int* p) {
   unsigned int v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -209,6 +216,36 @@ __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+
+// Resident launches, one lane: claims up to `want` published tickets from q on and
+// returns how many; -1 once the stop word is set or there was none for ring_idle_ns
+// (since wait_ns, 0 without a wait).  The words are read relaxed, and the queue only
+// when the tail has moved since the lane last found it used up (drained): an acquire
+// throws away the SM's L1 cache, which the paths beside a waiting warp live on, and
+// every waiting warp reads the same words.  Whoever gets a ticket acquires the tail.
+__device__ __forceinline__ int ring_claim(const LaunchCommon& c, int want, unsigned long long& q,
+                                          unsigned long long& wait_ns,
+                                          unsigned long long& drained) {
+  const unsigned long long pub = ld_relaxed_gpu(c.ring_tail);
+  if (pub != drained) {
+    unsigned long long cur = ld_relaxed_gpu(c.queue);
+    while (cur < pub) {  // (every retry means that another warp has claimed some)
+      const int n = (int)min((unsigned long long)want, pub - cur);
+      const unsigned long long was = atomicCAS(c.queue, cur, cur + n);
+      if (was == cur) {
+        q = cur;
+        wait_ns = 0;
+        return n;
+      }
+      cur = was;
+    }
+    drained = pub;
+  }
+  if (ld_relaxed_gpu(c.ring_stop)) return -1;
+  const unsigned long long now = global_ns();
+  if (wait_ns == 0) wait_ns = now;
+  return now - wait_ns > c.ring_idle_ns ? -1 : 0;
 }
 
 // max over the group of a double (butterfly over the group's L lanes)
@@ -259,15 +296,11 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
   // loop (COOP).  The whole warp stays in the loop until all of its groups
   // are out of work (M_IDLE), and that point holds the loop's only
   // warp-wide synchronisation, so every lane meets every other lane there.
-  // The resident-launch kernels (whose groups wait for tickets on their own)
-  // compute the same partial sums in the same order group by group (EP).
-  constexpr bool COOP_EVAL = MIXED && HOM::kCoop;
-  constexpr bool COOP = COOP_EVAL && !RING && !LOW;
+  constexpr bool COOP = MIXED && HOM::kCoop && !LOW;
   // Warps with several groups meet once per iteration and leave together (a
   // group out of work is M_IDLE until then): without that point the groups
   // drift apart and each runs the evaluation and the solve on its own.
-  constexpr bool MEET = groups_meet(L, RING, MIXED);
-  constexpr int EP = COOP_EVAL ? 32 / L : 1;
+  constexpr bool MEET = groups_meet(L, MIXED);
   constexpr int GL = L * HOM::WARPS;  // threads of a path
   const DevSettings& s = c.s;
   cx<R>* sb = reinterpret_cast<cx<R>*>(sm.sb);
@@ -295,6 +328,14 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
   bool be_bad = false;     // COOP: the endpoint failed the backward-error test
   unsigned long long ticket = 0;  // resident launches: the claimed ticket
   (void)ticket;
+  // resident launches: iterations since the group last looked for a ticket, when it
+  // first found none, the next nap
+  unsigned looks = 0, nap = 500;
+  unsigned long long wait_ns = 0, drained = ~0ull;
+  (void)looks;
+  (void)nap;
+  (void)wait_ns;
+  (void)drained;
   cx<double> xd = czero<double>();  // FP64 state
   cx<float> xf = czero<float>();    // FP32 state
   bool hi = !MIXED || PHASE == P_HIGH;  // the state lives in xd rather than xf
@@ -574,36 +615,6 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
       }
       mode = M_FETCH;
     }
-    if (RING && mode == M_FETCH) {
-      // resident launch: claim the next published ticket, or sleep and poll
-      // (bounded: the stop word or ring_idle_ns without work end the launch)
-      unsigned long long q = 0;
-      unsigned got = 0;
-      if (g.gl == 0) {
-        const unsigned long long t_wait = global_ns();
-        unsigned sleep_ns = 500;
-        for (;;) {
-          if (ld_relaxed_gpu(c.ring_stop)) break;
-          const unsigned long long pub = ld_acquire_gpu(c.ring_tail);
-          const unsigned long long cur = *reinterpret_cast<volatile unsigned long long*>(c.queue);
-          if (cur < pub) {
-            if (atomicCAS(c.queue, cur, cur + 1) == cur) {
-              q = cur;
-              got = 1;
-              break;
-            }
-            continue;
-          }
-          if (global_ns() - t_wait > c.ring_idle_ns) break;
-          __nanosleep(sleep_ns);  // back off while there is no work
-          sleep_ns = min(2u * sleep_ns, 32000u);
-        }
-      }
-      if (!__shfl_sync(g.mask, got, leader)) break;
-      ticket = __shfl_sync(g.mask, q, leader);
-      (void)ld_acquire_gpu(c.ring_tail);  // every lane: the slot's inputs are visible
-      item = (int64_t)(ticket % c.ring_items);
-    }
     if constexpr (PHASE == P_HIGH) {
       if (mode == M_FETCH && c.hand_list && !c.start_hi) {
         // the next path the low phase has handed over; with none on the list
@@ -648,7 +659,52 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         }
       }
     }
-    if (mode == M_FETCH) {
+    bool fetch = mode == M_FETCH;
+    if constexpr (RING) {
+      // Resident launch: the next published tickets.  Groups that share a warp look
+      // for them together, one lane for all, at once and then in every 16th iteration
+      // (the loads hold up the warp's paths), and wait inside the loop: a group that
+      // waits in a loop of its own holds up the warp's other groups with its naps.
+      // Both forms end with the stop word or after ring_idle_ns without work.
+      unsigned long long q = 0;
+      int got = 0, rank = 0;
+      if constexpr (MEET) {
+        const unsigned due =
+            __ballot_sync(0xffffffffu, g.gl == 0 && fetch && (looks & 15u) == 0u);
+        if (fetch) ++looks;
+        if (due != 0u) {
+          const int src = __ffs(due) - 1;
+          if (g.wl == src) got = ring_claim(c, __popc(due), q, wait_ns, drained);
+          got = __shfl_sync(0xffffffffu, got, src);
+          q = __shfl_sync(0xffffffffu, q, src);
+          drained = __shfl_sync(0xffffffffu, drained, src);
+          wait_ns = __shfl_sync(0xffffffffu, wait_ns, src);
+          const bool mine = (due >> leader & 1u) != 0u;
+          rank = __popc(due & ((1u << leader) - 1u));
+          if (mine && got < 0) mode = M_IDLE;
+          fetch = mine && rank < got;
+        } else {
+          fetch = false;
+        }
+      } else if (fetch) {
+        if (g.gl == 0)
+          while ((got = ring_claim(c, 1, q, wait_ns, drained)) == 0) {
+            __nanosleep(nap);  // back off while there is no work
+            nap = min(2u * nap, 32000u);
+          }
+        got = __shfl_sync(g.mask, got, leader);
+        q = __shfl_sync(g.mask, q, leader);
+        if (got < 0) break;
+      }
+      if (fetch) {
+        ticket = q + rank;
+        (void)ld_acquire_gpu(c.ring_tail);  // every lane: the slot's inputs are visible
+        item = (int64_t)(ticket % c.ring_items);
+        looks = 0;
+        nap = 500;
+      }
+    }
+    if (fetch) {
       bool stop = false;  // no further path for this group
       if (BUDGET && c.step_budget && !c.items) {
         // the budget stops new paths of the launch; started ones finish
@@ -788,6 +844,16 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
     if constexpr (MEET) {
       const unsigned live = __ballot_sync(0xffffffffu, g.gl == 0 && mode != M_IDLE);
       if (live == 0u) break;
+      if constexpr (RING) {
+        // nothing to track: back off, then look for tickets again
+        if (__ballot_sync(0xffffffffu, mode != M_IDLE && mode != M_FETCH) == 0u) {
+          __nanosleep(nap);
+          nap = min(2u * nap, 32000u);
+          looks = 0;
+          continue;
+        }
+        nap = 500;
+      }
     }
     if constexpr (COOP) {
       // Here the warp computes the groups' residuals one group at a time with
@@ -842,14 +908,14 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
         if (mode == M_REFINE || !res64) {
           cx<float> Hf;
           float sc;
-          hom.template residual_df<false, EP>(reinterpret_cast<const cdf*>(sm.vd), g.gl, te, Hf,
+          hom.template residual_df<false>(reinterpret_cast<const cdf*>(sm.vd), g.gl, te, Hf,
                                               sc);
           return cvt<R>(-Hf);
         }
       }
       cx<double> H64;
       double sc;
-      hom.template residual64<false, EP>(sm.vd, g.gl, te, 1.0 - te, H64, sc);
+      hom.template residual64<false>(sm.vd, g.gl, te, 1.0 - te, H64, sc);
       return cvt<R>(-H64);
     };
     bool sok;
@@ -1053,7 +1119,7 @@ __device__ __forceinline__ void run_phase(const PROB& prob, const LaunchCommon& 
           if constexpr (MIXED) {  // double-float residual: its error is ~2^-48 sc
             cx<float> Hf;
             float scf;
-            hom.template residual_df<true, EP>(reinterpret_cast<const cdf*>(sm.vd), g.gl, 1.0,
+            hom.template residual_df<true>(reinterpret_cast<const cdf*>(sm.vd), g.gl, 1.0,
                                                Hf, scf);
             r = (double)cabs2(Hf);
             sc = (double)scf;
@@ -1134,7 +1200,7 @@ template <int N, int L, bool MIXED, class PROB, class RE = double, int FORM = F_
 __device__ __forceinline__ void run_tracker(const PROB& prob, const LaunchCommon& c,
                                             const Group& g, const GroupMem& sm) {
   constexpr bool RING = FORM == F_RING;
-  if constexpr (FORM == F_BATCH && MIXED && groups_meet(L, RING, MIXED)) {
+  if constexpr (FORM == F_BATCH && MIXED && groups_meet(L, MIXED)) {
     if (!c.start_hi) {
       if (threadIdx.x == 0) *sm.hand = 0;
       __syncthreads();

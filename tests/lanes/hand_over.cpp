@@ -24,14 +24,14 @@ struct Straight {
     H = hc::mk<R>(R(x.re) - R(1 + ii) - t, R(0));
     Ht = hc::mk<R>(R(-1), R(0));
   }
-  template <bool SCALE, int EP = 1>
+  template <bool SCALE>
   __device__ void residual_df(const hc::cdf* xs, int i, double t, hc::cx<float>& H,
                               float& sc) const {
     const int ii = i < N ? i : 0;
     H = hc::mk<float>((float)((double)xs[ii].re() - 1.0 - ii - t), 0.f);
     sc = 4.f;
   }
-  template <bool SCALE, int EP = 1>
+  template <bool SCALE>
   __device__ void residual64(const hc::cx<double>* xs, int i, double t, double,
                              hc::cx<double>& H, double& sc) const {
     const int ii = i < N ? i : 0;

@@ -411,6 +411,7 @@ inline float2 __ffma2_rn(float2 a, float2 b, float2 c) {
 inline unsigned __float_as_uint(float f) { return lanes::unpack<unsigned>(lanes::pack(f)); }
 inline float __uint_as_float(unsigned u) { return lanes::unpack<float>(lanes::pack(u)); }
 inline float __int_as_float(int u) { return lanes::unpack<float>(lanes::pack(u)); }
+inline int __popc(unsigned v) { return __builtin_popcount(v); }
 inline int __ffs(unsigned v) { return __builtin_ffs((int)v); }
 inline float rsqrtf(float a) { return 1.0f / std::sqrt(a); }
 inline double __drcp_rn(double a) { return 1.0 / a; }

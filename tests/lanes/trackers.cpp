@@ -168,7 +168,7 @@ int family_rows(unsigned seed, int items) {
   return family<N>(seed, LS, 1, items, smem, hc::group_smem_bytes(L, 4, acc, eg) - 16,
                    [&](hc::TermArgs& a, unsigned char* mem) {
     return lanes::run(threads, seed, [&] {
-      const hc::Group g = hc::make_group<L, hc::groups_meet(L, false, MIXED)>();
+      const hc::Group g = hc::make_group<L, hc::groups_meet(L, MIXED)>();
       const hc::GroupMem sm = hc::make_group_mem<L>(mem, a.extra, acc, eg);
       hc::TermProblem<N, L, MIXED> prob{&a, g, sm};
       hc::run_tracker<N, L, MIXED, hc::TermProblem<N, L, MIXED>, double>(prob, a.c, g, sm);
@@ -207,7 +207,7 @@ int dense(unsigned seed, int items) {
   Block b(hc::block_smem_bytes(L, S::EXTRA, acc, threads, eg, XDF));
   lanes::atomic_word(b.mem + hc::group_smem_bytes(L, S::EXTRA, acc, eg, XDF) - 16);
   const int bad = lanes::run(threads, seed, [&] {
-    const hc::Group g = hc::make_group<L, hc::groups_meet(L, false, MIXED)>();
+    const hc::Group g = hc::make_group<L, hc::groups_meet(L, MIXED)>();
     const hc::GroupMem sm = hc::make_group_mem<L>(b.mem, S::EXTRA, acc, eg, XDF ? 1 : 0);
     hc::DenseProblem<N, DEG, L> prob{&a, sm, g.meet};
     hc::run_tracker<N, L, MIXED, hc::DenseProblem<N, DEG, L>, RE>(prob, a.c, g, sm);

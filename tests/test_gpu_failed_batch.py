@@ -29,9 +29,11 @@ def test_out_of_memory_beside_a_resident_launch():
     idle_s = 4.0
     s = hc.Stream(pr, slots=2, idle_us=int(idle_s * 1e6))
     try:
-        assert s.poll(s.submit(coef=coefs[0])) is not None  # the launch is resident now
+        assert s.poll(s.submit(coef=coefs[0])) is not None
+        ticket = s.submit(coef=coefs[0])  # the launch is resident until this is polled
         took = too_large()
         assert took < idle_s / 4, took
+        assert s.poll(ticket) is not None
     finally:
         s.close()
 
