@@ -628,8 +628,9 @@ hc_status hc_measure_fma_peak(int32_t fp64, int32_t iters, double* flops_per_s, 
  * allocator (it can synchronize the device), hosts whose allocator belongs to
  * another framework.  Runs the same dense total-degree kernels as
  * hc_track_batch on one batch, allocating nothing: every buffer besides the
- * caller's inputs and outputs lives in one fixed 16 MiB device array that
- * each GPU loading the library holds until exit.
+ * caller's inputs and outputs lives in one fixed 24 MiB device array (16 MiB for
+ * tables and lists, which bound the batch, 8 MiB for the links between the tracking
+ * loops) that each GPU loading the library holds until exit.
  *   n, degree   dense system: every monomial of degree <= degree in each of
  *               the n equations; degree 2 with n <= 12 or degree 3 with n <= 8
  *   gamma       host [2] unit-modulus homotopy constant

@@ -9,7 +9,8 @@
 //
 // The groups of a warp run the elimination in step (make_group): with group masks
 // each ran it on its own (batch 100,000, FP32, together with the staging below:
-// n = 4 12.6 -> 8.5 us, n = 8 31 -> 28, n = 20 327 -> 281; batch 1000, n = 8 6.0 -> 4.6).
+// n = 4 12.6 -> 8.5 us, n = 8 31 -> 28, n = 20 327 -> 281; batch 1000, n = 8, device time
+// of captured calls 4.1 -> 3.1; a call by itself takes 8 to 10 us either way, the host's).
 //
 // Data path: a block's systems are contiguous in A (row-major, system after
 // system), so the block stages them through shared memory with consecutive

@@ -87,7 +87,10 @@ struct Flow {
 // problem's last service time after its last start, and no longer than this: a
 // batch of several costs little more than one of one instance (the slowest path
 // sets the time), and an eighth is what a request can lose by it.  A problem that
-// is not in flight starts at once.
+// is not in flight starts at once.  Measured with / without: ten problems mixed at
+// 400/s p50 12.0-13.1 / 12.5-13.1 ms, p99 67-84 / 72-73, at 1000/s 57-61 / 58-61 and
+// 132-150 / 141-166; one kind (n = 8) at 8000/s 3.5 / 3.7: no faster, but a burst of a
+// few requests is sure to share batches, which it was not when batches became quick.
 constexpr auto kMostGather = std::chrono::milliseconds(4);
 
 }  // namespace
